@@ -1,7 +1,7 @@
 // Batched persistent launch: many independent SDDMM / SpMM problems of uneven
 // size in ONE kernel, each warp staging its gathers through a shared-memory
-// ring (ring.cuh).  Each item is cut into work units (one warp's worth of
-// balanced-schedule chunks, times the K blocks of an SpMM); a persistent grid
+// ring (ring.cuh, spmm_warp.cuh).  Each item is cut into work units (one chunk
+// of its balanced schedule, one warp's worth); a persistent grid
 // of one wave of CTAs pulls units off a device counter.  No warp ever waits on
 // another: split SpMM rows are finished by their last-arriving piece (see
 // spmm_impl.cuh), and the last warp to leave resets the counters, so the run
@@ -18,17 +18,15 @@ namespace spk {
 
 struct BatchDesc {
     int32_t op;      // 0 SDDMM, 1 SpMM
-    int32_t cls;     // (dtype, shape) class of the device routine
-    int32_t nkb;     // K blocks (SpMM)
-    int32_t gpw;     // lane groups per warp = 32 / G
+    int32_t cls;     // class of the device routine: SDDMM 8 * (BF16) + shape, SpMM 32 * (BF16) + vectors per row
     SddmmArgs sd;
     SpmmArgs sp;
 };
 
-// (G, NV, U) shapes available to batched items, per op; class = dtype * 8 +
-// position in the op's list.  Each (op, class) routine is a separate
-// non-inlined function, so the merged kernel needs no more registers than its
-// largest routine.
+// (G, NV, U) shapes accepted for batched items, per op.  SDDMM runs the shape;
+// SpMM has one layout per row width (spmm_warp.cuh) and only checks it.  Each
+// routine is a separate non-inlined function, so the merged kernel needs no
+// more registers than its largest routine.
 #define SPK_BATCH_SDDMM_SHAPES(X) \
     X(0, 4, 1, 4)                 \
     X(1, 8, 1, 4)                 \
@@ -58,9 +56,11 @@ constexpr int kBatchThreads = 128;
 
 // Shared-memory ring of one warp for one (op, shape); a batch gives every warp
 // the largest ring among its items' shapes.
-static int batch_ring_bytes(int op, const Shape& sh)
+static int batch_ring_bytes(int op, const Shape& sh, int cl)
 {
-    const int b = op == 0 ? sddmm_ring_bytes(sh.G, sh.NV, sh.U, 2) : spmm_ring_bytes(sh.NV, sh.U);
+    const int b = op == 0 ? sddmm_ring_bytes(sh.G, sh.NV, sh.U, 2)
+                          : (cl <= 4 ? SpmmWarp<DT_F32, 4>::bytes(1) : (cl <= 8 ? SpmmWarp<DT_F32, 8>::bytes(1)
+                                                                                 : SpmmWarp<DT_F32, 16>::bytes(1)));
     return (b + 127) / 128 * 128;
 }
 
@@ -75,23 +75,16 @@ __device__ __noinline__ void batch_sddmm_unit(const SddmmArgs& a, int64_t unit, 
     else sddmm_ring_span<DT, G, NV, U, 2, false>(a, threadIdx.x & 31, wsm, b0.y, b1.y);
 }
 
-// SpMM: one chunk per lane group, 32/G consecutive chunks per unit.
-template <int DT, int G, int NV, int U>
-__device__ __noinline__ void batch_spmm_unit(const SpmmArgs& a, int64_t unit, int nkb, unsigned char* wsm)
+// SpMM: one chunk per warp (spmm_warp.cuh), rows of at most CL 16-byte vectors.
+template <int DT, int CL>
+__device__ __noinline__ void batch_spmm_unit(const SpmmArgs& a, int64_t c, unsigned char* wsm)
 {
-    const Group<G> g;
-    const int kb = (int)(unit % nkb);
-    const int64_t c = (unit / nkb) * (32 / G) + ((threadIdx.x & 31) / G);
     if (c >= a.nchunks) return;
     const int2 b0 = a.bnd[c], b1 = a.bnd[c + 1];
     const int4 m = a.meta[c];
-    if (b1.y == b0.y && m.z < b0.x) return;
     const int hs0 = (m.x >= 0) ? __ldg(a.head_s0 + c) : -1;
-    uint4* wring = reinterpret_cast<uint4*>(wsm);
-    if (a.K / vec_elems(DT) >= (kb + 1) * G * NV)
-        spmm_ring_span<DT, G, NV, U, true>(a, g, wring, kb, nkb, b0.x, b0.y, b1.x, b1.y, m, hs0);
-    else
-        spmm_ring_span<DT, G, NV, U, false>(a, g, wring, kb, nkb, b0.x, b0.y, b1.x, b1.y, m, hs0);
+    if (a.K * dt_bytes(DT) == CL * 16) spmm_warp_span<DT, CL, SPMM_STORE, true>(a, wsm, 0, 1, b0, b1, m, hs0);
+    else spmm_warp_span<DT, CL, SPMM_STORE, false>(a, wsm, 0, 1, b0, b1, m, hs0);
 }
 
 // MINB: CTAs per SM the register budget is cut for (6: 80 registers; 5: 96
@@ -128,11 +121,12 @@ __global__ void __launch_bounds__(kBatchThreads, MINB) k_batch(const BatchDesc* 
             }
         } else {
             switch (cls) {
-#define X(i, G_, NV_, U_)                                                           \
-    case i: batch_spmm_unit<DT_F32, G_, NV_, U_>(d.sp, local, d.nkb, wsm); break;   \
-    case 8 + i: batch_spmm_unit<DT_BF16, G_, NV_, U_>(d.sp, local, d.nkb, wsm); break;
-                SPK_BATCH_SPMM_SHAPES(X)
-#undef X
+            case 4: batch_spmm_unit<DT_F32, 4>(d.sp, local, wsm); break;
+            case 8: batch_spmm_unit<DT_F32, 8>(d.sp, local, wsm); break;
+            case 16: batch_spmm_unit<DT_F32, 16>(d.sp, local, wsm); break;
+            case 32 + 4: batch_spmm_unit<DT_BF16, 4>(d.sp, local, wsm); break;
+            case 32 + 8: batch_spmm_unit<DT_BF16, 8>(d.sp, local, wsm); break;
+            case 32 + 16: batch_spmm_unit<DT_BF16, 16>(d.sp, local, wsm); break;
             }
         }
         __syncwarp();
@@ -244,15 +238,13 @@ static spk_status plan_batch(const spk_batch_item* items, int32_t count, BatchPl
             if (list[q].G == G && list[q].NV == NV && list[q].U == U) sidx = q;
         if (sidx < 0 || G * NV < nvec)
             return bfail(SPK_ERR_UNSUPPORTED, where + "shape not available in batched mode");
-        const int rb = batch_ring_bytes(it.op, list[sidx]);
+        const int cl = nvec <= 4 ? 4 : (nvec <= 8 ? 8 : 16);         // SpMM: 16-byte vectors per gathered row
+        const int rb = batch_ring_bytes(it.op, list[sidx], cl);
         if (rb > P.ring_bytes) P.ring_bytes = rb;
         if (list[sidx].U > 4 || it.dt == SPK_BF16) P.wide = true;
         BatchDesc& d = P.descs[m];
         d.op = it.op;
-        d.cls = (it.dt == SPK_BF16 ? 8 : 0) + sidx;
-        d.gpw = 32 / G;
-        d.nkb = 1;
-        const int64_t wunits = (S->nchunks + d.gpw - 1) / d.gpw;
+        d.cls = it.op == 0 ? (it.dt == SPK_BF16 ? 8 : 0) + sidx : (it.dt == SPK_BF16 ? 32 : 0) + cl;
         if (it.op == 0) {
             SddmmArgs& a = d.sd;
             a.M = S->M; a.N = S->N; a.nnz = S->nnz; a.K = it.K;
@@ -264,7 +256,6 @@ static spk_status plan_batch(const spk_batch_item* items, int32_t count, BatchPl
             a.bnd = S->bnd; a.nchunks = S->nchunks;
             P.unit_begin[m + 1] = units + (S->nnz > 0 ? S->nchunks : 0);     // one chunk per warp
         } else {
-            d.nkb = (nvec + G * NV - 1) / (G * NV);
             SpmmArgs& a = d.sp;
             a.M = S->M; a.N = S->N; a.nnz = S->nnz; a.K = it.K;
             a.rowptr = S->rowptr; a.colidx = S->colidx; a.rowidx = S->rowidx; a.vperm = nullptr;
@@ -277,7 +268,7 @@ static spk_status plan_batch(const spk_batch_item* items, int32_t count, BatchPl
             a.nchunks = S->nchunks;
             P.carry_off[m] = carry;
             carry += align256((size_t)S->npieces * it.K * 4);
-            P.unit_begin[m + 1] = units + (S->M > 0 ? wunits * d.nkb : 0);
+            P.unit_begin[m + 1] = units + (S->M > 0 ? S->nchunks : 0);              // one chunk per warp
         }
         units = P.unit_begin[m + 1];
     }

@@ -39,6 +39,33 @@ __device__ __forceinline__ void cpa4(void* smem, const void* gmem)
                  : "memory");
 }
 
+// Two floats in one 64-bit register pair, as the packed FMA takes them.
+typedef unsigned long long f32x2;
+__device__ __forceinline__ void ffma2(f32x2& acc, f32x2 s, f32x2 x)
+{
+    asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc) : "l"(s), "l"(x));
+}
+__device__ __forceinline__ f32x2 pack2(uint32_t lo, uint32_t hi)
+{
+    f32x2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "r"(lo), "r"(hi));
+    return r;
+}
+__device__ __forceinline__ float lo2(f32x2 x) { return __uint_as_float((uint32_t)x); }
+__device__ __forceinline__ float hi2(f32x2 x) { return __uint_as_float((uint32_t)(x >> 32)); }
+
+// 16-byte asynchronous copy under a predicate, without a branch.
+__device__ __forceinline__ void cpa16_if(bool p, unsigned smem, const void* gmem)
+{
+    asm volatile("{\n .reg .pred p;\n setp.ne.b32 p, %2, 0;\n @p cp.async.cg.shared.global [%0], [%1], 16;\n}\n"
+                 ::"r"(smem), "l"(gmem), "r"((int)p)
+                 : "memory");
+}
+__device__ __forceinline__ void cpa16_at(unsigned smem, const void* gmem)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(smem), "l"(gmem) : "memory");
+}
+
 // Shared memory of one SDDMM warp with D batch slots, in bytes (host and
 // device): B slots, A slots, then rows / values / second values / batch
 // metadata per slot, rounded up to 128 bytes so that every warp's slots stay
@@ -408,281 +435,9 @@ __device__ __forceinline__ void sddmm_ring_span(const SddmmArgs& a, int lane, un
     cp_async_wait<0>();
 }
 
-// ----------------------------------------------------------------------------
-// SpMM (Eq. 2): a lane group walks its own span (chunk) of the balanced
-// schedule, accumulating K-slices of the current output row in registers, as
-// in the register path; gathered rows arrive through the warp's ring (two
-// slots).  Each group streams its own index tiles of 4G entries: the columns
-// one tile ahead in registers (they address the gathers), the COO rows and
-// values by cp.async into a double-buffered tile in shared memory (they are
-// only read by the compute).  A full batch that stays in the current row
-// takes the fast path (no per-nonzero checks); span edges and row changes go
-// nonzero by nonzero, flushing finished rows.  Values must be absent or
-// 16-byte aligned without a second factor or a slot permutation (other calls
-// take the register path).
-// ----------------------------------------------------------------------------
-// VB: bytes of one lane vector, 16, or 8 for 16-bit operands spread over
-// twice the lanes (a group of G lanes then covers G * NV * VB bytes of a row).
-// Per warp: two batch slots of gathered rows, the staged COO rows (two tiles
-// of 128 entries) and the staged values (two tiles per head).
-__host__ __device__ constexpr int spmm_ring_bytes(int NV, int U, int VB = 16, int heads = 1)
-{
-    return 2 * U * NV * 32 * VB + 2 * 128 * 4 + heads * 2 * 128 * 4;
-}
-
-__device__ __forceinline__ void cpa8(void* smem, const void* gmem)
-{
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"((unsigned)__cvta_generic_to_shared(smem)),
-                 "l"(gmem)
-                 : "memory");
-}
-
-template <int VB>
-struct LaneVec { using type = uint4; };
-template <>
-struct LaneVec<8> { using type = uint2; };
-
-template <int DT, int VECN>
-__device__ __forceinline__ void unpack_vec(const uint4 v, float (&f)[VECN])
-{
-    Raw<DT, VECN> r;
-    r.w[0] = v.x; r.w[1] = v.y; r.w[2] = v.z; r.w[3] = v.w;
-    unpack_all<DT, VECN>(r, f);
-}
-template <int DT, int VECN>
-__device__ __forceinline__ void unpack_vec(const uint2 v, float (&f)[VECN])
-{
-    Raw<DT, VECN> r;
-    r.w[0] = v.x; r.w[1] = v.y;
-    unpack_all<DT, VECN>(r, f);
-}
-
-template <int DT, int G, int NV, int U, bool ALLV, int VB = 16>
-__device__ __forceinline__ void spmm_ring_span(const SpmmArgs& a, const Group<G>& g, uint4* wring16, int kb, int nkb,
-                                               int r0, int e0, int r1, int e1, const int4 meta, int head_s0)
-{
-    static_assert(VB == 16 || (VB == 8 && DT != DT_F32 && DT != DT_E4M3), "8-byte lane vectors are for 16-bit operands");
-    using Vec = typename LaneVec<VB>::type;
-    constexpr int VECN = VB / dt_bytes(DT);
-    Vec* wring = reinterpret_cast<Vec*>(wring16);
-    constexpr int TG = 4 * G;                       // entries per group tile (one int4 per lane)
-    static_assert(U % 4 == 0 && TG % U == 0 && TG / U >= 2, "batches must tile the group tile");
-    const int gl = g.gl;
-    const int lane = threadIdx.x & 31;
-    const int grp = lane / G;
-    const int nvec = a.K / VECN;
-    const int vbase = kb * G * NV;
-    bool vin[NV];
-#pragma unroll
-    for (int t = 0; t < NV; ++t) vin[t] = ALLV || (vbase + t * G + gl < nvec);
-    const char* __restrict__ Bb = reinterpret_cast<const char*>(a.B) + (vbase + gl) * VB;
-    const unsigned ldb_bytes = (unsigned)a.ldb * dt_bytes(DT);
-    const float* __restrict__ vals = a.vals;
-    // tile buffers after the B slots: rows[2][128] then vals[2][128] per warp;
-    // group grp owns entries [grp * 4G, (grp + 1) * 4G) of each 128-entry buffer
-    int* trow = reinterpret_cast<int*>(wring + 2 * U * NV * 32) + grp * TG;
-    float* tval = reinterpret_cast<float*>(reinterpret_cast<int*>(wring + 2 * U * NV * 32) + 2 * 128) + grp * TG;
-    // several heads (NV = 1): head h's values in the h-th pair of value tiles;
-    // this lane reads the tiles of the head its columns belong to
-    float* tval_l = tval;
-    if (a.heads > 1) tval_l += min((vbase + gl) / (nvec / a.heads), a.heads - 1) * 256;
-
-    float acc[NV][VECN];
-#pragma unroll
-    for (int t = 0; t < NV; ++t)
-#pragma unroll
-        for (int q = 0; q < VECN; ++q) acc[t][q] = 0.f;
-    int cur = r0;
-    auto flush = [&](int row) {
-        if (row == r0 && meta.x >= 0)
-            finish_piece<VECN, G, NV>(a, g, kb, nkb, nvec, meta.x, head_s0, row, acc);
-        else if (row == r1 && meta.y >= 0)
-            finish_piece<VECN, G, NV>(a, g, kb, nkb, nvec, meta.y, meta.y, row, acc);
-        else
-            write_row<VECN, G, NV>(a, g, kb, nvec, row, acc);
-    };
-
-    if (e0 < e1) {
-        const int tb0 = e0 & ~3;
-        const int nb = (e1 - tb0 + U - 1) / U;
-        auto cols = [&](int t) -> int4 {
-            const int e = tb0 + t * TG + 4 * gl;
-            if (e + 4 <= e1) return ld4(a.colidx + e);
-            int4 c = make_int4(0, 0, 0, 0);
-            if (e < e1) c.x = __ldg(a.colidx + e);
-            if (e + 1 < e1) c.y = __ldg(a.colidx + e + 1);
-            if (e + 2 < e1) c.z = __ldg(a.colidx + e + 2);
-            return c;
-        };
-        auto stage_tile = [&](int t) {             // rows and values of tile t into buffer t & 1
-            const int e = tb0 + t * TG + 4 * gl;
-            const int n = e1 - e;
-            if (n <= 0) return;
-            const int bytes = n >= 4 ? 16 : 4 * n;
-            const int o = (t & 1) * 128 + 4 * gl;
-            cp_async16(trow + o, a.rowidx + e, bytes);
-            if (vals) {
-                if (a.heads == 1) {
-                    cp_async16(tval + o, vals + e, bytes);
-                } else {
-                    for (int h = 0; h < a.heads; ++h) {
-                        const float* hv = vals + (int64_t)h * a.hstride + e;
-                        if ((a.hstride & 3) == 0) {
-                            cp_async16(tval + h * 256 + o, hv, bytes);
-                        } else {                    // a head array off 16-byte alignment: four 4-byte copies
-                            const int n4 = n >= 4 ? 4 : n;
-                            for (int q = 0; q < n4; ++q) cpa4(tval + h * 256 + o + q, hv + q);
-                        }
-                    }
-                }
-            }
-        };
-        int4 tc = cols(0), nc = cols(1);
-        int itile = 0;
-        stage_tile(0);
-        auto issue = [&](int b) {
-            if (b < nb) {
-                const int t = (b * U) / TG;
-                if (t != itile) {
-                    tc = nc;
-                    nc = cols(t + 1);
-                    stage_tile(t);
-                    itile = t;
-                }
-                const int src0 = ((b * U) % TG) >> 2;
-                int j[U];
-#pragma unroll
-                for (int c = 0; c < U / 4; ++c) {
-                    j[4 * c + 0] = __shfl_sync(g.mask, tc.x, src0 + c, G);
-                    j[4 * c + 1] = __shfl_sync(g.mask, tc.y, src0 + c, G);
-                    j[4 * c + 2] = __shfl_sync(g.mask, tc.z, src0 + c, G);
-                    j[4 * c + 3] = __shfl_sync(g.mask, tc.w, src0 + c, G);
-                }
-                const int eb = tb0 + b * U;
-                Vec* sl = wring + (b & 1) * U * NV * 32 + lane;
-                auto copy_row = [&](int u) {
-                    const char* brow = Bb + (size_t)(unsigned)j[u] * ldb_bytes;
-#pragma unroll
-                    for (int t2 = 0; t2 < NV; ++t2)
-                        if (vin[t2]) {
-                            if constexpr (VB == 16) cpa16(sl + (u * NV + t2) * 32, brow + t2 * G * 16);
-                            else cpa8(sl + (u * NV + t2) * 32, brow + t2 * G * 8);
-                        }
-                };
-                if constexpr (DT == DT_F32 && U >= 8) {
-                    if (eb >= e0 && eb + U <= e1) {     // whole batch inside the span: no per-entry guard
-#pragma unroll
-                        for (int u = 0; u < U; ++u) copy_row(u);
-                    } else {
-#pragma unroll
-                        for (int u = 0; u < U; ++u)
-                            if (eb + u >= e0 && eb + u < e1) copy_row(u);
-                    }
-                } else {                                // 16-bit rows, short batches: one guarded loop
-                    const bool full = (eb >= e0) && (eb + U <= e1);
-#pragma unroll
-                    for (int u = 0; u < U; ++u) {
-                        if (!full && (eb + u < e0 || eb + u >= e1)) continue;
-                        copy_row(u);
-                    }
-                }
-            }
-            cp_async_commit();
-        };
-
-        issue(0);
-        for (int b = 0; b < nb; ++b) {
-            __syncwarp(g.mask);
-            issue(b + 1);
-            cp_async_wait<1>();
-            __syncwarp(g.mask);
-            const int eb = tb0 + b * U;
-            const Vec* sl = wring + (b & 1) * U * NV * 32 + lane;
-            const int o = (((b * U) / TG) & 1) * 128 + (b * U) % TG;
-            int rc[U];
-            float sc[U];
-#pragma unroll
-            for (int c = 0; c < U / 4; ++c) {
-                const int4 r4 = *reinterpret_cast<const int4*>(trow + o + 4 * c);
-                rc[4 * c + 0] = r4.x; rc[4 * c + 1] = r4.y; rc[4 * c + 2] = r4.z; rc[4 * c + 3] = r4.w;
-                if (vals) {
-                    const float4 v4 = *reinterpret_cast<const float4*>(tval_l + o + 4 * c);
-                    sc[4 * c + 0] = v4.x; sc[4 * c + 1] = v4.y; sc[4 * c + 2] = v4.z; sc[4 * c + 3] = v4.w;
-                } else {
-                    sc[4 * c + 0] = sc[4 * c + 1] = sc[4 * c + 2] = sc[4 * c + 3] = 1.f;
-                }
-            }
-            // one fast/general decision for the lane groups running together
-            // (each group walks its own span, so they may have parted): a batch
-            // that could take the fast path is also right on the general one,
-            // and groups running the two paths one after the other cost both
-            if (__all_sync(__activemask(), eb >= e0 && eb + U <= e1 && rc[U - 1] == cur)) {
-#pragma unroll
-                for (int u = 0; u < U; ++u)
-#pragma unroll
-                    for (int t = 0; t < NV; ++t) {
-                        if (!vin[t]) continue;
-                        float bf[VECN];
-                        unpack_vec<DT, VECN>(sl[(u * NV + t) * 32], bf);
-                        axpy_pairs<VECN>(acc[t], sc[u], bf);
-                    }
-            } else if constexpr (DT == DT_F32 && U >= 8) {
-                // a row ends inside the batch, or the batch straddles the
-                // span's ends: one copy of the row-change code, entries read
-                // back from the staged tiles by a runtime index (measured
-                // 3 % faster for FP32 rows in batches of 8; 7 % slower for
-                // 16-bit rows and 14 % slower for FP32 batches of 4)
-                const int u0 = max(e0 - eb, 0), u1 = min(e1 - eb, U);
-#pragma unroll 1
-                for (int u = u0; u < u1; ++u) {
-                    const int r = trow[o + u];
-                    if (r != cur) {
-                        flush(cur);
-                        for (int rr = cur + 1; rr < r; ++rr) zero_row<VECN, G, NV>(a, g, kb, nvec, rr);
-                        cur = r;
-#pragma unroll
-                        for (int t = 0; t < NV; ++t)
-#pragma unroll
-                            for (int q = 0; q < VECN; ++q) acc[t][q] = 0.f;
-                    }
-                    const float sv = vals ? tval_l[o + u] : 1.f;
-#pragma unroll
-                    for (int t = 0; t < NV; ++t) {
-                        if (!vin[t]) continue;
-                        float bf[VECN];
-                        unpack_vec<DT, VECN>(sl[(u * NV + t) * 32], bf);
-                        axpy_pairs<VECN>(acc[t], sv, bf);
-                    }
-                }
-            } else {
-#pragma unroll
-                for (int u = 0; u < U; ++u) {
-                    const int e = eb + u;
-                    if (e < e0 || e >= e1) continue;
-                    if (rc[u] != cur) {
-                        flush(cur);
-                        for (int rr = cur + 1; rr < rc[u]; ++rr) zero_row<VECN, G, NV>(a, g, kb, nvec, rr);
-                        cur = rc[u];
-#pragma unroll
-                        for (int t = 0; t < NV; ++t)
-#pragma unroll
-                            for (int q = 0; q < VECN; ++q) acc[t][q] = 0.f;
-                    }
-#pragma unroll
-                    for (int t = 0; t < NV; ++t) {
-                        if (!vin[t]) continue;
-                        float bf[VECN];
-                        unpack_vec<DT, VECN>(sl[(u * NV + t) * 32], bf);
-                        axpy_pairs<VECN>(acc[t], sc[u], bf);
-                    }
-                }
-            }
-        }
-        cp_async_wait<0>();
-        __syncwarp(g.mask);
-    }
-    flush(cur);
-    for (int rr = cur + 1; rr <= meta.z; ++rr) zero_row<VECN, G, NV>(a, g, kb, nvec, rr);
-}
+// Shared memory of one warp of a lane-group span with two batch slots: the
+// gathered rows (U rows of NV 16-byte vectors a lane), the staged COO rows and
+// the staged values (two tiles of 128 entries each).
+__host__ __device__ constexpr int spmm_ring_bytes(int NV, int U) { return 2 * U * NV * 32 * 16 + 4 * 128 * 4; }
 
 }  // namespace spk

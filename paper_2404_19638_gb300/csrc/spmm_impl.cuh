@@ -17,112 +17,10 @@
 // by the schedule, so results are bitwise reproducible.
 #pragma once
 #include "ring.cuh"
+#include "rows.cuh"
+#include "spmm_warp.cuh"
 
 namespace spk {
-
-template <int VECN>
-__device__ __forceinline__ void write_vec(const SpmmArgs& a, int64_t idx, const float* v)
-{
-    float o[VECN];
-#pragma unroll
-    for (int q = 0; q < VECN; ++q) o[q] = v[q];
-    switch (a.dtc) {
-    case DT_BF16:
-        if (a.accumulate) {
-            float old[VECN];
-            load_elems_cg<DT_BF16, VECN>(a.C, idx, old);
-#pragma unroll
-            for (int q = 0; q < VECN; ++q) o[q] += old[q];
-        }
-        store_elems<DT_BF16, VECN>(a.C, idx, o);
-        break;
-    case DT_F16:
-        if (a.accumulate) {
-            float old[VECN];
-            load_elems_cg<DT_F16, VECN>(a.C, idx, old);
-#pragma unroll
-            for (int q = 0; q < VECN; ++q) o[q] += old[q];
-        }
-        store_elems<DT_F16, VECN>(a.C, idx, o);
-        break;
-    default:
-        if (a.accumulate) {
-            float old[VECN];
-            load_elems_cg<DT_F32, VECN>(a.C, idx, old);
-#pragma unroll
-            for (int q = 0; q < VECN; ++q) o[q] += old[q];
-        }
-        store_elems<DT_F32, VECN>(a.C, idx, o);
-    }
-}
-
-template <int VECN, int G, int NV>
-__device__ __forceinline__ void write_row(const SpmmArgs& a, const Group<G>& g, int kb, int nvec, int64_t row,
-                                          const float (&acc)[NV][VECN])
-{
-#pragma unroll
-    for (int t = 0; t < NV; ++t) {
-        const int v = kb * G * NV + t * G + g.gl;
-        if (v < nvec) write_vec<VECN>(a, row * a.ldc + (int64_t)v * VECN, acc[t]);
-    }
-}
-
-template <int VECN, int G, int NV>
-__device__ __forceinline__ void zero_row(const SpmmArgs& a, const Group<G>& g, int kb, int nvec, int64_t row)
-{
-    if (a.accumulate) return;
-    float z[VECN];
-#pragma unroll
-    for (int q = 0; q < VECN; ++q) z[q] = 0.f;
-#pragma unroll
-    for (int t = 0; t < NV; ++t) {
-        const int v = kb * G * NV + t * G + g.gl;
-        if (v < nvec) write_vec<VECN>(a, row * a.ldc + (int64_t)v * VECN, z);
-    }
-}
-
-// Deposit one piece of a split row and, if it is the last to arrive, finish the row.
-template <int VECN, int G, int NV>
-__device__ __forceinline__ void finish_piece(const SpmmArgs& a, const Group<G>& g, int kb, int nkb, int nvec,
-                                             int slot, int s0, int64_t row, const float (&acc)[NV][VECN])
-{
-#pragma unroll
-    for (int t = 0; t < NV; ++t) {
-        const int v = kb * G * NV + t * G + g.gl;
-        if (v < nvec) store_elems<DT_F32, VECN>(a.carry, (int64_t)slot * a.K + (int64_t)v * VECN, acc[t]);
-    }
-    __threadfence();
-    __syncwarp(g.mask);
-    int last = 0;
-    if (g.gl == 0) {
-        const int np = __ldcg(a.slot_np + s0);
-        const int old = atomicAdd(a.cnt + s0, 1);
-        last = (old == np * nkb - 1);
-    }
-    last = __shfl_sync(g.mask, last, 0, G);
-    if (!last) return;
-    __threadfence();
-    const int np = __ldcg(a.slot_np + s0);
-    for (int kb2 = 0; kb2 < nkb; ++kb2) {
-#pragma unroll
-        for (int t = 0; t < NV; ++t) {
-            const int v = kb2 * G * NV + t * G + g.gl;
-            if (v >= nvec) continue;
-            float sum[VECN];
-#pragma unroll
-            for (int q = 0; q < VECN; ++q) sum[q] = 0.f;
-            for (int sl = s0; sl < s0 + np; ++sl) {
-                float x[VECN];
-                load_elems_cg<DT_F32, VECN>(a.carry, (int64_t)sl * a.K + (int64_t)v * VECN, x);
-#pragma unroll
-                for (int q = 0; q < VECN; ++q) sum[q] += x[q];
-            }
-            write_vec<VECN>(a, row * a.ldc + (int64_t)v * VECN, sum);
-        }
-    }
-    __syncwarp(g.mask);
-    if (g.gl == 0) atomicExch(a.cnt + s0, 0);   // ready for the next launch
-}
 
 template <int DTB, int VECN, int G, int NV, int U, bool KNOWN_ROW>
 __device__ __forceinline__ void spmm_span(const SpmmArgs& a, const Group<G>& g, int* tiles, int kb, int nkb,
@@ -283,39 +181,6 @@ __global__ void __launch_bounds__(256, VECN > 1 ? (U * NV <= 4 ? 4 : (U * NV <= 
     }
 }
 
-// Ring path: one group per span of the balanced schedule, gathered rows
-// staged in the warp's shared-memory ring (ring.cuh).
-template <int DT, int G, int NV, int U, int VB>
-__global__ void __launch_bounds__(RING_THREADS, ring_min_ctas(spmm_ring_bytes(NV, U, VB))) k_spmm_ring(const SpmmArgs a)
-{
-    extern __shared__ __align__(16) unsigned char ring_smem[];
-    const Group<G> g;
-    uint4* wring = reinterpret_cast<uint4*>(ring_smem) + (threadIdx.x >> 5) * (spmm_ring_bytes(NV, U, VB, a.heads) / 16);
-    const int kb = blockIdx.y, nkb = gridDim.y;
-    const int64_t ngroups = (int64_t)gridDim.x * blockDim.x / G;
-    const int64_t gid = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / G;
-    const bool allv = a.K / (VB / dt_bytes(DT)) >= (kb + 1) * G * NV;
-    for (int64_t c = gid; c < a.nchunks; c += ngroups) {
-        const int2 b0 = a.bnd[c], b1 = a.bnd[c + 1];
-        const int4 m = a.meta[c];
-        if (b1.y == b0.y && m.z < b0.x) continue;          // nothing in this chunk
-        const int hs0 = (m.x >= 0) ? __ldg(a.head_s0 + c) : -1;
-        if (allv) spmm_ring_span<DT, G, NV, U, true, VB>(a, g, wring, kb, nkb, b0.x, b0.y, b1.x, b1.y, m, hs0);
-        else spmm_ring_span<DT, G, NV, U, false, VB>(a, g, wring, kb, nkb, b0.x, b0.y, b1.x, b1.y, m, hs0);
-    }
-}
-
-template <int DT, int VB>
-inline const void* spmm_ring_kernel_for(int shape)
-{
-    switch (shape) {
-#define X(i, G_, NV_, U_) case i: return (const void*)&k_spmm_ring<DT, G_, NV_, U_, VB>;
-        SPK_SHAPES(X)
-#undef X
-    }
-    return nullptr;
-}
-
 template <int DTB, int VECN>
 inline const void* spmm_kernel_for(int shape)
 {
@@ -338,33 +203,7 @@ cudaError_t launch_spmm_t(const Launch& L, const SpmmArgs& a, cudaStream_t s)
     const int nkb = (nvec + sh.G * sh.NV - 1) / (sh.G * sh.NV);
     const int64_t items = a.bnd ? a.nchunks : a.M;
     if (items <= 0) return cudaSuccess;
-    if constexpr (DTB != DT_E4M3) {
-        const bool ring_ok = L.vec && L.ring && a.bnd && !a.vperm && !a.vals2 && (!a.vals || a.vals_staged) &&
-                             (a.heads == 1 || shape_at(L.shape).NV == 1);
-        if (ring_ok) {
-            // 16-bit operands whose 16-byte vectors would leave half the group's
-            // lanes idle are spread over all of them as 8-byte vectors
-            constexpr bool can_half = (DTB == DT_BF16 || DTB == DT_F16);
-            const bool half = can_half && 2 * nvec <= sh.G * sh.NV && a.K % 4 == 0;
-            const int vb = half ? 8 : 16;
-            const void* rf = half ? spmm_ring_kernel_for<DTB, (can_half ? 8 : 16)>(L.shape)
-                                  : spmm_ring_kernel_for<DTB, 16>(L.shape);
-            if (!rf) return cudaErrorInvalidValue;
-            const int nkb2 = half ? (a.K / 4 + sh.G * sh.NV - 1) / (sh.G * sh.NV) : nkb;
-
-            const int64_t groups_per_cta = RING_THREADS / sh.G;
-            int64_t blocks = (items + groups_per_cta - 1) / groups_per_cta;
-            if (blocks > 0x7fffffffLL) blocks = 0x7fffffffLL;
-            if (nkb2 > 65535) return cudaErrorInvalidValue;
-            const size_t smem = (size_t)(RING_THREADS / 32) * spmm_ring_bytes(sh.NV, sh.U, vb, a.heads);
-            if (smem > 48 * 1024) {
-                cudaError_t e = cudaFuncSetAttribute(rf, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-                if (e != cudaSuccess) return e;
-            }
-            void* args[] = {(void*)&a};
-            return cudaLaunchKernel(rf, dim3((unsigned)blocks, (unsigned)nkb2), dim3(RING_THREADS), args, smem, s);
-        }
-    }
+    if (L.vec && L.ring && a.bnd) return launch_spmm_warp<DTB>(a, s);
     const int64_t groups_per_cta = L.threads / sh.G;
     int64_t blocks = (items + groups_per_cta - 1) / groups_per_cta;
     if (blocks > 0x7fffffffLL) blocks = 0x7fffffffLL;
