@@ -1,6 +1,6 @@
 // Batched persistent launch: many independent SDDMM / SpMM problems of uneven
 // size in ONE kernel, each warp staging its gathers through a shared-memory
-// ring (ring.cuh, spmm_warp.cuh).  Each item is cut into work units (one chunk
+// ring (sddmm_warp.cuh, spmm_warp.cuh).  Each item is cut into work units (one chunk
 // of its balanced schedule, one warp's worth); a persistent grid
 // of one wave of CTAs pulls units off a device counter.  No warp ever waits on
 // another: split SpMM rows are finished by their last-arriving piece (see
@@ -58,21 +58,20 @@ constexpr int kBatchThreads = 128;
 // the largest ring among its items' shapes.
 static int batch_ring_bytes(int op, const Shape& sh, int cl)
 {
-    const int b = op == 0 ? sddmm_ring_bytes(sh.G, sh.NV, sh.U, 2)
+    const int b = op == 0 ? sddmm_warp_bytes(sh.G, sh.NV, sh.U)
                           : (cl <= 4 ? SpmmWarp<DT_F32, 4>::bytes(1) : (cl <= 8 ? SpmmWarp<DT_F32, 8>::bytes(1)
                                                                                  : SpmmWarp<DT_F32, 16>::bytes(1)));
     return (b + 127) / 128 * 128;
 }
 
-// SDDMM: one chunk per warp (groups take interleaved batches of it), gathered
-// rows through the warp's ring (ring.cuh).
+// SDDMM: one chunk per warp (sddmm_warp.cuh).
 template <int DT, int G, int NV, int U>
 __device__ __noinline__ void batch_sddmm_unit(const SddmmArgs& a, int64_t unit, unsigned char* wsm)
 {
     if (unit >= a.nchunks) return;
-    const int2 b0 = a.bnd[unit], b1 = a.bnd[unit + 1];
-    if (a.K / vec_elems(DT) >= G * NV) sddmm_ring_span<DT, G, NV, U, 2, true>(a, threadIdx.x & 31, wsm, b0.y, b1.y);
-    else sddmm_ring_span<DT, G, NV, U, 2, false>(a, threadIdx.x & 31, wsm, b0.y, b1.y);
+    const int e0 = a.bnd[unit].y, n = a.bnd[unit + 1].y - e0;
+    if (a.K / vec_elems(DT) >= G * NV) sddmm_warp_chunk<DT, DT, G, NV, U, true>(a, wsm, e0, n);
+    else sddmm_warp_chunk<DT, DT, G, NV, U, false>(a, wsm, e0, n);
 }
 
 // SpMM: one chunk per warp (spmm_warp.cuh), rows of at most CL 16-byte vectors.

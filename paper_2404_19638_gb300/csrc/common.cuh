@@ -52,6 +52,32 @@ __device__ __forceinline__ float unpack_one(const uint32_t* w, int k)
     }
 }
 
+// E4M3 codes -> floats, through FP16 (exact).  The halves are taken apart in
+// PTX: through the header's 16-bit types every pair costs two byte permutes
+// more (SDDMM with E4M3 rows of 128: 0.478 ms, 0.261 without them).
+__device__ __forceinline__ void e4m3x4_to_f16x2(uint32_t w, uint32_t& lo, uint32_t& hi)
+{
+    asm("{\n .reg .b16 l, h;\n mov.b32 {l, h}, %2;\n cvt.rn.f16x2.e4m3x2 %0, l;\n cvt.rn.f16x2.e4m3x2 %1, h;\n}"
+        : "=r"(lo), "=r"(hi) : "r"(w));
+}
+__device__ __forceinline__ void f16x2_to_f32(uint32_t w, float& lo, float& hi)
+{
+    asm("{\n .reg .b16 l, h;\n mov.b32 {l, h}, %2;\n cvt.f32.f16 %0, l;\n cvt.f32.f16 %1, h;\n}"
+        : "=f"(lo), "=f"(hi) : "r"(w));
+}
+template <int N>
+__device__ __forceinline__ void e4m3_to_f32(const uint32_t* w, float* out)
+{
+    static_assert(N % 2 == 0, "pairs");
+#pragma unroll
+    for (int k = 0; k < N; k += 4) {
+        uint32_t lo, hi;
+        e4m3x4_to_f16x2(w[k >> 2], lo, hi);
+        f16x2_to_f32(lo, out[k], out[k + 1]);
+        if (k + 2 < N) f16x2_to_f32(hi, out[k + 2], out[k + 3]);
+    }
+}
+
 template <int DT, int N>
 __device__ __forceinline__ void load_elems(const void* base, int64_t idx, float* out)
 {
@@ -76,14 +102,7 @@ __device__ __forceinline__ void load_elems(const void* base, int64_t idx, float*
         w[0] = __ldg(reinterpret_cast<const unsigned char*>(p));
     }
     if constexpr (DT == DT_E4M3 && N >= 2) {
-#pragma unroll
-        for (int k = 0; k < N; k += 2) {
-            uint32_t x = w[k >> 2];
-            __nv_fp8x2_storage_t q2 = (__nv_fp8x2_storage_t)((x >> (8 * (k & 3))) & 0xffffu);
-            __half2_raw hr = __nv_cvt_fp8x2_to_halfraw2(q2, __NV_E4M3);
-            float2 f = __half22float2(__half2(hr));
-            out[k] = f.x; out[k + 1] = f.y;
-        }
+        e4m3_to_f32<N>(w, out);
     } else {
 #pragma unroll
         for (int k = 0; k < N; ++k) out[k] = unpack_one<DT>(w, k);
@@ -164,14 +183,7 @@ template <int DT, int N>
 __device__ __forceinline__ void unpack_all(const Raw<DT, N>& r, float* out)
 {
     if constexpr (DT == DT_E4M3 && N >= 2) {
-#pragma unroll
-        for (int k = 0; k < N; k += 2) {
-            const uint32_t x = r.w[k >> 2];
-            const __nv_fp8x2_storage_t q2 = (__nv_fp8x2_storage_t)((x >> (8 * (k & 3))) & 0xffffu);
-            const __half2_raw hr = __nv_cvt_fp8x2_to_halfraw2(q2, __NV_E4M3);
-            const float2 f = __half22float2(__half2(hr));
-            out[k] = f.x; out[k + 1] = f.y;
-        }
+        e4m3_to_f32<N>(r.w, out);
     } else {
 #pragma unroll
         for (int k = 0; k < N; ++k) out[k] = unpack_one<DT>(r.w, k);

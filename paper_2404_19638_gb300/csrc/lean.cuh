@@ -115,6 +115,9 @@ __device__ __forceinline__ void sddmm_warp_span(const SddmmArgs& a, int lane, in
             if (a.vals) sv = __ldg(a.vals + ew);
             if (a.vals2) sv *= __ldg(a.vals2 + ew);
         }
+        float scl = 1.f;                                 // row scales, applied once per finished dot
+        if constexpr (DTA == DT_E4M3)
+            if (writer) scl = __ldg(a.a_scale + (KNOWN_ROW ? r0 : __ldg(a.rowidx + ew))) * __ldg(a.b_scale + __ldg(a.colidx + ew));
         float p[U];
 #pragma unroll
         for (int u = 0; u < U; ++u) {
@@ -132,7 +135,6 @@ __device__ __forceinline__ void sddmm_warp_span(const SddmmArgs& a, int lane, in
                 dot_pairs<VECN>(acc, av[t], bf);
             }
             p[u] = acc.x + acc.y;
-            if constexpr (DTA == DT_E4M3) p[u] *= __ldg(a.a_scale + cur) * __ldg(a.b_scale + j[u]);
         }
         // Reduce-scatter over the low log2(U) lane bits, then butterflies over
         // the remaining G/U lane subsets: nonzero eg + (gl % U) ends in lane gl.
@@ -148,7 +150,7 @@ __device__ __forceinline__ void sddmm_warp_span(const SddmmArgs& a, int lane, in
         }
 #pragma unroll
         for (int d = U; d < G; d <<= 1) p[0] += __shfl_xor_sync(gmask, p[0], d, G);
-        if (writer) __stcs(a.out + ew, sv * p[0]);
+        if (writer) __stcs(a.out + ew, sv * (DTA == DT_E4M3 ? p[0] * scl : p[0]));
     }
 }
 

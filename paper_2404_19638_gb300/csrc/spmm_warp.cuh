@@ -245,13 +245,12 @@ __device__ __forceinline__ void spmm_warp_span(const SpmmArgs& a, unsigned char*
             }
             constexpr int STEP = BLK ? W::RBB : W::EPI * W::RBB;
             if (FULL && left >= U) {
-#pragma unroll
-                for (int i = 0; i < NS; ++i) cpa16_at(slot + i * STEP, Bb + (size_t)(unsigned)j[i] * ldb_bytes);
+                for_const<NS>([&](auto i) { cpa16_at<i.value * STEP>(slot, Bb + (size_t)(unsigned)j[i.value] * ldb_bytes); });
             } else {
-#pragma unroll
-                for (int i = 0; i < NS; ++i)
-                    cpa16_if(vin && (BLK ? sub * NS + i : i * W::EPI + sub) < left, slot + i * STEP,
-                             Bb + (size_t)(unsigned)j[i] * ldb_bytes);
+                for_const<NS>([&](auto i) {
+                    cpa16_if<i.value * STEP>(vin && (BLK ? sub * NS + i.value : i.value * W::EPI + sub) < left, slot,
+                                             Bb + (size_t)(unsigned)j[i.value] * ldb_bytes);
+                });
             }
         }
         cp_async_commit();
