@@ -542,6 +542,13 @@ extern "C" spk_status spk_spmm_workspace_size(spk_csr S, int32_t K, size_t* byte
     return SPK_OK;
 }
 
+// 16-byte vectors throughout: whole vectors a row, aligned rows of B and C.
+static bool spmm_vec(spk_dtype dtb, const void* B, int64_t ldb, int32_t K, spk_dtype dtc, const void* C, int64_t ldc)
+{
+    return (K % vec_elems(dtb)) == 0 && aligned16(B) && aligned16(C) && (ldb * dt_bytes(dtb)) % 16 == 0 &&
+           (ldc * dt_bytes(dtc)) % 16 == 0;
+}
+
 static spk_status spmm_common(const char* name, const spk_csr_s* S, const float* vals, const float* vals2,
                               spk_dtype dtb, const void* B, int64_t ldb, const float* b_scale, int32_t K,
                               spk_dtype dtc, void* C, int64_t ldc, int32_t accumulate, void* ws, size_t ws_bytes,
@@ -560,8 +567,7 @@ static spk_status spmm_common(const char* name, const spk_csr_s* S, const float*
     REQUIRE(dtb != SPK_E4M3 || b_scale, SPK_ERR_ARG, "%s: E4M3 input needs row scales", name);
     if (S->M == 0) return SPK_OK;
     const int vecn = vec_elems(dtb);
-    const bool vec = (K % vecn) == 0 && aligned16(B) && aligned16(C) && (ldb * dt_bytes(dtb)) % 16 == 0 &&
-                     (ldc * dt_bytes(dtc)) % 16 == 0;
+    const bool vec = spmm_vec(dtb, B, ldb, K, dtc, C, ldc);
     Launch L;
     spk_status st;
     if (heads > 1) {
@@ -1125,6 +1131,13 @@ extern "C" spk_status spk_spmm_t_workspace_size(spk_tplan P, int32_t K, size_t* 
     return SPK_OK;
 }
 
+static bool spmm_t_gathers_values(const spk_tplan_s* P, spk_dtype dty, const void* Y, int64_t ldy, int32_t K,
+                                  spk_dtype dtx, const void* X, int64_t ldx, const spk_tune* tune)
+{
+    const int variant = (tune && tune->variant) ? tune->variant : (P->St.has_sched ? 2 : 1);
+    return variant == 2 && spmm_vec(dty, Y, ldy, K, dtx, X, ldx);
+}
+
 extern "C" spk_status spk_spmm_t(spk_tplan P, const float* vals, const float* vals2, spk_dtype dty, const void* Y,
                                  int64_t ldy, const float* y_scale, int32_t K, spk_dtype dtx, void* X, int64_t ldx,
                                  int32_t accumulate, void* workspace, size_t ws_bytes, const spk_tune* tune,
@@ -1146,14 +1159,16 @@ extern "C" spk_status spk_spmm_t(spk_tplan P, const float* vals, const float* va
                                 nullptr, dty, Y, ldy, y_scale, K, dtx, X, ldx, accumulate, w ? w + vb : nullptr,
                                 w ? ws_bytes - vb : 0, tune, (cudaStream_t)stream, true, true);
     if (st != SPK_OK) return st;
-    const float* vt = nullptr;
-    if ((vals || vals2) && P->St.nnz > 0) {
-        float* out = reinterpret_cast<float*>(w);
-        cudaError_t e = launch_permute_vals(P->perm, vals, vals2, P->St.nnz, out, (cudaStream_t)stream);
-        if (e != cudaSuccess) return cuda_fail(e, "spk_spmm_t value permutation");
-        vt = out;
-    }
-    return spmm_common("spk_spmm_t", &P->St, vt, nullptr, dty, Y, ldy, y_scale, K, dtx, X, ldx, accumulate,
+    // The balanced 16-byte vector path gathers the values through the
+    // permutation where it loads an index tile; every other path reads them
+    // from the workspace in CSC slot order.
+    if (!(vals || vals2) || P->St.nnz == 0 || spmm_t_gathers_values(P, dty, Y, ldy, K, dtx, X, ldx, tune))
+        return spmm_common("spk_spmm_t", &P->St, vals, vals2, dty, Y, ldy, y_scale, K, dtx, X, ldx, accumulate,
+                           w ? w + vb : nullptr, w ? ws_bytes - vb : 0, tune, (cudaStream_t)stream);
+    float* out = reinterpret_cast<float*>(w);
+    cudaError_t e = launch_permute_vals(P->perm, vals, vals2, P->St.nnz, out, (cudaStream_t)stream);
+    if (e != cudaSuccess) return cuda_fail(e, "spk_spmm_t value permutation");
+    return spmm_common("spk_spmm_t", &P->St, out, nullptr, dty, Y, ldy, y_scale, K, dtx, X, ldx, accumulate,
                        w ? w + vb : nullptr, w ? ws_bytes - vb : 0, tune, (cudaStream_t)stream, true);
 }
 

@@ -184,8 +184,9 @@ __device__ __forceinline__ void spmm_warp_span(const SpmmArgs& a, unsigned char*
     if (a.heads > 1) tval_l += min(col0 / (a.K / a.heads), a.heads - 1) * 64;
     const bool plain = a.vals && !a.vals2 && !a.vperm && a.heads == 1 && DT != DT_E4M3;
 
-    int nc = 0, nr = 0;
+    int nc = 0, nr = 0, np = 0;
     float nv = 1.f;
+    if (a.vperm && lane < n) np = __ldg(a.vperm + e0 + lane);
     auto load_tile = [&](int i) {                                   // entry i of the chunk into this lane's registers
         if (i >= n) return;
         const int e = e0 + i;
@@ -194,9 +195,10 @@ __device__ __forceinline__ void spmm_warp_span(const SpmmArgs& a, unsigned char*
         if (plain) {
             nv = __ldg(a.vals + e);
         } else if (a.heads == 1) {
-            const int vi = a.vperm ? __ldg(a.vperm + e) : e;
+            const int vi = a.vperm ? np : e;                        // a permuted slot was loaded one tile before
             nv = a.vals ? __ldg(a.vals + vi) : 1.f;
             if (a.vals2) nv *= __ldg(a.vals2 + vi);
+            if (a.vperm && i + 32 < n) np = __ldg(a.vperm + e + 32);
             if constexpr (DT == DT_E4M3) nv *= __ldg(a.b_scale + nc);
         }
     };

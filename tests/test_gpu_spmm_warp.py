@@ -100,3 +100,20 @@ def test_infinities_and_nan_stay_in_their_rows(spk):
     assert torch.equal(torch.isnan(C), torch.isnan(R)) and torch.equal(torch.isinf(C), torch.isinf(R))
     fin = torch.isfinite(R)
     torch.testing.assert_close(C[fin], R[fin], rtol=1e-5, atol=1e-4)
+
+
+@pytest.mark.parametrize("dt,K", [("f32", 32), ("bf16", 64), ("e4m3", 48), ("f32", 260)])
+@pytest.mark.parametrize("both", [False, True])
+def test_transpose_gathers_values_through_the_plan(spk, dt, K, both):
+    """S^T Y takes the values through the slot permutation while it loads its
+    index tiles; the register path reads them permuted into the workspace."""
+    M, N = 330, 401
+    rp, ci = edge_pattern(M, N, K + 5, long_row=900)
+    g = np.random.default_rng(K)
+    S = spk.CSR(rp, ci, (M, N), device=DEV, chunk_work=64)
+    P = S.transpose_plan(64)
+    Y, s, _, _ = _factor(spk, dt, M, K, g)
+    v = [torch.from_numpy(g.uniform(-1, 1, ci.size).astype(np.float32)).to(DEV) for _ in range(2)]
+    args = (v[0], v[1]) if both else (None, v[1])
+    got = [spk.spmm_t(S, Y, *args, y_scale=s, plan=P, tune=t) for t in (None, {"variant": 3})]
+    assert torch.equal(got[0], got[1])
