@@ -320,6 +320,19 @@ spk_status spk_fused_rowdot(int64_t M, int32_t K, int32_t heads, const float* dY
 spk_status spk_fused_score_grad(spk_csr S, int32_t heads, int32_t softmax, float scale, const float* vals,
                                 const float* w, const float* dw, const float* rowdot, float* c, void* stream);
 
+/* The row side of the FusedMM backward in one pass over S: dw = <dY_i, B_j>
+ * per head, w and c as above (scores, lse: the forward's; rowdot from
+ * spk_fused_rowdot; lse and rowdot only with softmax), dA_i = sum_j c B_j.
+ * cw receives nnz x heads pairs (c, w), 8-byte aligned, for spk_spmm_t_pair.
+ * dA and dY are FP32.  Workspace: spk_fusedmm_workspace_size.  Covers rows of
+ * B of at most 512 bytes, 16-byte aligned operands and row strides, one head
+ * or heads whose columns fill a power of two of lanes; SPK_ERR_UNSUPPORTED
+ * otherwise (nothing is launched). */
+spk_status spk_fused_grad(spk_csr S, const float* scores, const float* lse, const float* rowdot, const float* vals,
+                          float scale, int32_t softmax, spk_dtype dtb, const void* B, int64_t ldb, const float* dY,
+                          int64_t lddy, int32_t K, int32_t heads, float* dA, int64_t ldda, float* cw,
+                          void* workspace, size_t ws_bytes, void* stream);
+
 /* --------------------------------------------- tensor-core dense tiles -- */
 /* Where a 128-row x 64-column tile of S holds many entries, its SDDMM (Eq. 1)
  * is a real contraction: the tile's A panel (128 x K) and B tile (64 x K) are
@@ -398,6 +411,16 @@ spk_status spk_spmm_t_mh_workspace_size(spk_tplan P, int32_t K, int32_t heads, s
 spk_status spk_spmm_t_mh(spk_tplan P, const float* vals, int64_t hstride, int32_t heads, spk_dtype dty, const void* Y,
                          int64_t ldy, int32_t K, float* X, int64_t ldx, int32_t accumulate, void* workspace,
                          size_t ws_bytes, void* stream);
+
+/* The column side of the FusedMM backward: X (N x K, FP32) (+)= S_c^T A +
+ * S_w^T Y, the pairs (c, w) of spk_fused_grad gathered through the plan's
+ * permutation.  Y is FP32.  Workspace: one row of K floats per piece of a
+ * split row of S^T (spk_spmm_t_workspace_size covers it).  16-byte aligned
+ * operands and row strides, head widths of whole 16-byte vectors of A, at most
+ * 64 heads; SPK_ERR_UNSUPPORTED otherwise. */
+spk_status spk_spmm_t_pair(spk_tplan P, const float* cw, int32_t heads, spk_dtype dta, const void* A, int64_t lda,
+                           const float* Y, int64_t ldy, int32_t K, float* X, int64_t ldx, int32_t accumulate,
+                           void* workspace, size_t ws_bytes, void* stream);
 
 /* ----------------------------------------------------------- precision -- */
 /* Round-to-nearest-even casts of n FP32 values to BF16 or F16. */

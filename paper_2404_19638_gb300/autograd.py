@@ -106,10 +106,16 @@ class GNNLayerFunction(torch.autograd.Function):
         S = ctx.S
         dY = dY.contiguous().float()
         v = _vals_or_none(vals)
-        dE = ops.sddmm(S, dY, H, use_default_vals=False)
-        acc = ops.spmm(S, H, v, dE, use_default_vals=False)
-        ops.spmm_t(S, H, v, dE, out=acc, accumulate=True, use_default_vals=False)
-        ops.spmm_t(S, dY, e, out=acc, accumulate=True, use_default_vals=False)
+        try:                                       # (dE, (S.dE) H) in one pass over S, the two S^T products in another
+            acc, ee = ops.fused_grad(S, H, dY, e.reshape(1, -1), None, None, 1, False, 1.0, v)
+            ops.spmm_t_pair(S, ee, H, dY, out=acc, accumulate=True)
+        except SpkError as err:
+            if err.code != "SPK_ERR_UNSUPPORTED":
+                raise
+            dE = ops.sddmm(S, dY, H, use_default_vals=False)
+            acc = ops.spmm(S, H, v, dE, use_default_vals=False)
+            ops.spmm_t(S, H, v, dE, out=acc, accumulate=True, use_default_vals=False)
+            ops.spmm_t(S, dY, e, out=acc, accumulate=True, use_default_vals=False)
         dH = acc if H.dtype == torch.float32 else ops.cast(acc, H.dtype)
         return None, None, dH
 
@@ -126,6 +132,32 @@ def _dw_per_head(S, dY, B, dw, heads, Kh):
         ops.sddmm(S, dY[:, c0:c0 + Kh], B[:, c0:c0 + Kh], out=dw[h], use_default_vals=False)
 
 
+def _fused_backward_steps(S, v, A, B, scores, lse, dY, R, heads, scale, softmax, need_dB):
+    """dA and dB (FP32; dB None where not needed) in separate passes: dw by one
+    multi-head SDDMM (FP32 operands; one SDDMM per head otherwise, or where no
+    multi-head kernel covers K), the score gradient c, dA = one multi-head
+    SpMM, dB = two multi-head SpMM^T."""
+    Kh = A.size(1) // heads
+    w = ops.fused_weights(S, scores, lse, heads, softmax) if softmax else scores
+    dw = torch.empty_like(scores)
+    if B.dtype == torch.float32 and heads > 1:
+        try:                                       # all heads in one pass over the pattern
+            ops.sddmm_mh(S, dY, B, heads, out=dw)
+        except SpkError as err:                    # no multi-head kernel for this K: one SDDMM per head
+            if err.code != "SPK_ERR_UNSUPPORTED":
+                raise
+            _dw_per_head(S, dY, B, dw, heads, Kh)
+    else:
+        _dw_per_head(S, dY, B, dw, heads, Kh)
+    c = ops.fused_score_grad(S, w, dw, R, heads, softmax, scale, v)
+    dA = ops.spmm_mh(S, B, c, heads)
+    dB = None
+    if need_dB:
+        dB = ops.spmm_t_mh(S, A, c, heads)
+        ops.spmm_t_mh(S, dY, w, heads, out=dB, accumulate=True)
+    return dA, dB
+
+
 class FusedMMFunction(torch.autograd.Function):
     """Differentiable FusedMM: per head h, e = scale * s * <A_i, B_j>,
     w = e or its row softmax, Y_i = sum_j w_ij B_j.
@@ -135,12 +167,11 @@ class FusedMMFunction(torch.autograd.Function):
           = <dY_i, Y_i> (read from the saved output)
       c = scale * s * g;  dA = C B;  dB = C^T A + W^T dY  (C, W: S's pattern
       holding c, w)
-    Steps: dw by one multi-head SDDMM (FP32 operands; one SDDMM per head
-    otherwise, or where no multi-head kernel covers K), the row term and score gradient
-    kernels (c folds in the sparse values, so every SpMM takes one value
-    array per head), then dA = one multi-head SpMM (c per head) and
-    dB = two multi-head SpMM^T (c with A, then w with dY added), each one
-    pass over the pattern for all heads, in FP32.  The sparse values are not
+    Steps: the row term; one pass over S that gathers B once for dw, the
+    weights, c and dA (ops.fused_grad); one pass over S^T that adds both
+    products of dB to one output (ops.spmm_t_pair), all heads at once, in
+    FP32.  Where those kernels don't cover K, the heads or the alignment, the
+    same steps one by one (_fused_backward_steps).  The sparse values are not
     differentiated.
     """
 
@@ -159,31 +190,18 @@ class FusedMMFunction(torch.autograd.Function):
         S, heads, scale, softmax = ctx.S, ctx.heads, ctx.scale, ctx.softmax
         dY = dY.contiguous().float()
         v = _vals_or_none(vals)
-        K = A.size(1)
-        Kh = K // heads
-        w = ops.fused_weights(S, scores, lse, heads, softmax) if softmax else scores
-        dw = torch.empty_like(scores)
-        if B.dtype == torch.float32 and heads > 1:
-            try:                                   # all heads in one pass over the pattern
-                ops.sddmm_mh(S, dY, B, heads, out=dw)
-            except SpkError as err:                # no multi-head kernel for this K: one SDDMM per head
-                if err.code != "SPK_ERR_UNSUPPORTED":
-                    raise
-                _dw_per_head(S, dY, B, dw, heads, Kh)
-        else:
-            _dw_per_head(S, dY, B, dw, heads, Kh)
+        need_dB = ctx.needs_input_grad[3]
         R = ops.fused_rowdot(dY, Y, heads) if softmax else None
-        c = ops.fused_score_grad(S, w, dw, R, heads, softmax, scale, v)
-        dA = dB = None
-        if ctx.needs_input_grad[2]:
-            dA = ops.spmm_mh(S, B, c, heads)
-            if A.dtype != torch.float32:
-                dA = ops.cast(dA, A.dtype)
-        if ctx.needs_input_grad[3]:
-            dB = ops.spmm_t_mh(S, A, c, heads)
-            ops.spmm_t_mh(S, dY, w, heads, out=dB, accumulate=True)
-            if B.dtype != torch.float32:
-                dB = ops.cast(dB, B.dtype)
+        try:
+            dA, cw = ops.fused_grad(S, B, dY, scores, lse, R, heads, softmax, scale, v)
+            dB = ops.spmm_t_pair(S, cw, A, dY) if need_dB else None
+        except SpkError as err:                    # no one-pass kernels for this K and these heads
+            if err.code != "SPK_ERR_UNSUPPORTED":
+                raise
+            dA, dB = _fused_backward_steps(S, v, A, B, scores, lse, dY, R, heads, scale, softmax, need_dB)
+        dA = None if not ctx.needs_input_grad[2] else dA if A.dtype == torch.float32 else ops.cast(dA, A.dtype)
+        if dB is not None and B.dtype != torch.float32:
+            dB = ops.cast(dB, B.dtype)
         return None, None, dA, dB, None, None, None
 
 

@@ -91,6 +91,10 @@ _PROTOS = {
     "spk_fused_weights": (ctypes.c_int, [_vp, _i32, _i32, _vp, _vp, _vp, _vp]),
     "spk_fused_rowdot": (ctypes.c_int, [_i64, _i32, _i32, _vp, _i64, _vp, _i64, _vp, _vp]),
     "spk_fused_score_grad": (ctypes.c_int, [_vp, _i32, _i32, ctypes.c_float, _vp, _vp, _vp, _vp, _vp, _vp]),
+    "spk_fused_grad": (ctypes.c_int, [_vp, _vp, _vp, _vp, _vp, ctypes.c_float, _i32, ctypes.c_int, _vp, _i64, _vp,
+                                      _i64, _i32, _i32, _vp, _i64, _vp, _vp, _sz, _vp]),
+    "spk_spmm_t_pair": (ctypes.c_int, [_vp, _vp, _i32, ctypes.c_int, _vp, _i64, _vp, _i64, _i32, _vp, _i64, _i32,
+                                       _vp, _sz, _vp]),
     "spk_tc_plan_size": (ctypes.c_int, [_vp, _i32, _i32, _P(_sz), _P(_sz)]),
     "spk_tc_plan_build": (ctypes.c_int, [_vp, _i32, _i32, _vp, _sz, _vp, _sz, _P(_vp), _vp]),
     "spk_tc_plan_info": (ctypes.c_int, [_vp, _P(_i64), _P(_i64), _P(_i64)]),

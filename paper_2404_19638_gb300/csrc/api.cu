@@ -9,6 +9,7 @@
 
 #include "common.cuh"
 #include "fused.cuh"
+#include "pair.cuh"
 #include "heads.cuh"
 
 namespace spk {
@@ -703,9 +704,10 @@ extern "C" spk_status spk_fusedmm(spk_csr S, const float* vals, float scale, int
     } else if (dt != SPK_F32 && heads >= 4 && mh_fits(2)) {
         mh_nv = 2;
     }
+    const bool warp = !shaped && !mh_asked && fused_warp_supported(dt, K, heads);
     const bool mh = mh_asked || (!shaped && !one_head && mh_fits(mh_nv));
     int G, NV = 1, U = 4, idx = -1;
-    if (!mh) {
+    if (!mh && !warp) {
         if (nvh <= 4) G = 4;
         else if (nvh <= 8) G = 8;
         else if (nvh <= 16) G = 16;
@@ -734,11 +736,14 @@ extern "C" spk_status spk_fusedmm(spk_csr S, const float* vals, float scale, int
     a.softmax = softmax; a.scale = scale;
     a.rowptr = S->rowptr; a.colidx = S->colidx; a.rowidx = S->rowidx; a.vals = vals;
     a.A = A; a.lda = lda; a.B = B; a.ldb = ldb; a.Y = Y; a.ldy = ldy; a.scores = scores; a.lse = lse;
+    a.rowdot = nullptr; a.cw = nullptr;
     a.bnd = S->bnd; a.meta = S->meta; a.head_s0 = S->head_s0; a.slot_np = S->slot_np; a.cnt = S->cnt;
     a.carry = reinterpret_cast<float*>(workspace);
     a.nchunks = S->nchunks;
     cudaError_t e;
-    if (mh) {
+    if (warp) {
+        e = launch_fused_warp(dt, a, (cudaStream_t)stream);
+    } else if (mh) {
         e = launch_fused_mh_nv(dt, nv / mh_nv, mh_nv, a, (cudaStream_t)stream);
     } else {
         Launch L;
@@ -746,6 +751,52 @@ extern "C" spk_status spk_fusedmm(spk_csr S, const float* vals, float scale, int
         e = launch_fused(dt, L, a, (cudaStream_t)stream);
     }
     if (e != cudaSuccess) return cuda_fail(e, "spk_fusedmm");
+    return SPK_OK;
+}
+
+extern "C" spk_status spk_fused_grad(spk_csr S, const float* scores, const float* lse, const float* rowdot,
+                                     const float* vals, float scale, int32_t softmax, spk_dtype dtb, const void* B,
+                                     int64_t ldb, const float* dY, int64_t lddy, int32_t K, int32_t heads, float* dA,
+                                     int64_t ldda, float* cw, void* workspace, size_t ws_bytes, void* stream)
+{
+    REQUIRE(S, SPK_ERR_ARG, "spk_fused_grad: S is NULL");
+    REQUIRE(!S->vperm, SPK_ERR_ARG, "spk_fused_grad: pattern belongs to a transpose plan");
+    REQUIRE(S->has_sched, SPK_ERR_UNSUPPORTED, "spk_fused_grad: needs spk_schedule_build first");
+    REQUIRE(dtb == SPK_F32 || dtb == SPK_BF16 || dtb == SPK_F16, SPK_ERR_DTYPE,
+            "spk_fused_grad: B must be F32, BF16 or F16");
+    REQUIRE(K >= 1 && heads >= 1 && K % heads == 0, SPK_ERR_SHAPE,
+            "spk_fused_grad: K (%d) must be a multiple of heads (%d)", K, heads);
+    REQUIRE(softmax == 0 || softmax == 1, SPK_ERR_ARG, "spk_fused_grad: softmax must be 0 or 1");
+    REQUIRE(ldb >= K && lddy >= K && ldda >= K, SPK_ERR_SHAPE, "spk_fused_grad: leading dimensions must be >= K");
+    REQUIRE(stride32(ldb, dtb) && stride32(lddy, SPK_F32), SPK_ERR_SHAPE,
+            "spk_fused_grad: row strides must be below 4 GiB");
+    REQUIRE(S->nnz == 0 || (B && dY && scores && cw && (!softmax || (lse && rowdot))), SPK_ERR_ARG,
+            "spk_fused_grad: NULL array");
+    REQUIRE(S->M == 0 || dA, SPK_ERR_ARG, "spk_fused_grad: dA is NULL");
+    REQUIRE((K / heads) % vec_elems(dtb) == 0 && fused_warp_supported(dtb, K, heads), SPK_ERR_UNSUPPORTED,
+            "spk_fused_grad: no kernel for K = %d in %d heads", K, heads);
+    REQUIRE(aligned16(B) && aligned16(dY) && aligned16(dA) && (ldb * dt_bytes(dtb)) % 16 == 0 && lddy % 4 == 0 &&
+                ldda % 4 == 0 && (reinterpret_cast<uintptr_t>(cw) & 7u) == 0,
+            SPK_ERR_UNSUPPORTED, "spk_fused_grad: B, dY, dA must be 16-byte aligned with 16-byte row strides");
+    const size_t need = (size_t)S->npieces * (((size_t)K + 2 * (size_t)heads + 3) / 4 * 4) * 4;
+    if (need > 0) {
+        REQUIRE(workspace && ws_bytes >= need, SPK_ERR_WORKSPACE, "spk_fused_grad: workspace has %zu bytes, needs %zu",
+                workspace ? ws_bytes : (size_t)0, need);
+        REQUIRE(aligned16(workspace), SPK_ERR_WORKSPACE, "spk_fused_grad: workspace must be 16-byte aligned");
+    }
+    if (S->M == 0) return SPK_OK;
+    FusedArgs a;
+    a.M = S->M; a.N = S->N; a.nnz = S->nnz; a.K = K; a.heads = heads; a.dh = K / heads;
+    a.softmax = softmax; a.scale = scale;
+    a.rowptr = S->rowptr; a.colidx = S->colidx; a.rowidx = S->rowidx; a.vals = vals;
+    a.A = dY; a.lda = lddy; a.B = B; a.ldb = ldb; a.Y = dA; a.ldy = ldda;
+    a.scores = const_cast<float*>(scores); a.lse = const_cast<float*>(lse);      // read only in the backward
+    a.rowdot = rowdot; a.cw = cw;
+    a.bnd = S->bnd; a.meta = S->meta; a.head_s0 = S->head_s0; a.slot_np = S->slot_np; a.cnt = S->cnt;
+    a.carry = reinterpret_cast<float*>(workspace);
+    a.nchunks = S->nchunks;
+    cudaError_t e = launch_fused_grad(dtb, a, (cudaStream_t)stream);
+    if (e != cudaSuccess) return cuda_fail(e, "spk_fused_grad");
     return SPK_OK;
 }
 
@@ -1216,6 +1267,48 @@ extern "C" spk_status spk_spmm_t_mh(spk_tplan P, const float* vals, int64_t hstr
         }
     return spmm_common("spk_spmm_t_mh", &P->St, vt, nullptr, dty, Y, ldy, nullptr, K, SPK_F32, X, ldx, accumulate,
                        w + vb, ws_bytes - vb, nullptr, (cudaStream_t)stream, true, false, heads, ws_stride);
+}
+
+extern "C" spk_status spk_spmm_t_pair(spk_tplan P, const float* cw, int32_t heads, spk_dtype dta, const void* A,
+                                      int64_t lda, const float* Y, int64_t ldy, int32_t K, float* X, int64_t ldx,
+                                      int32_t accumulate, void* workspace, size_t ws_bytes, void* stream)
+{
+    REQUIRE(P, SPK_ERR_ARG, "spk_spmm_t_pair: P is NULL");
+    REQUIRE(heads >= 1 && K >= 1 && K % heads == 0, SPK_ERR_SHAPE,
+            "spk_spmm_t_pair: K (%d) must be a multiple of heads (%d)", K, heads);
+    REQUIRE(accumulate == 0 || accumulate == 1, SPK_ERR_ARG, "spk_spmm_t_pair: accumulate must be 0 or 1");
+    REQUIRE(dta == SPK_F32 || dta == SPK_BF16 || dta == SPK_F16, SPK_ERR_DTYPE,
+            "spk_spmm_t_pair: A must be F32, BF16 or F16");
+    REQUIRE(lda >= K && ldy >= K && ldx >= K, SPK_ERR_SHAPE, "spk_spmm_t_pair: leading dimensions must be >= K");
+    REQUIRE(stride32(lda, dta) && stride32(ldy, SPK_F32), SPK_ERR_SHAPE,
+            "spk_spmm_t_pair: row strides must be below 4 GiB");
+    const spk_csr_s& T = P->St;
+    REQUIRE(T.has_sched, SPK_ERR_UNSUPPORTED, "spk_spmm_t_pair: the plan has no schedule");
+    REQUIRE(T.nnz == 0 || (cw && A && Y), SPK_ERR_ARG, "spk_spmm_t_pair: NULL array");
+    REQUIRE(T.M == 0 || X, SPK_ERR_ARG, "spk_spmm_t_pair: X is NULL");
+    // a lane's columns (up to 4) belong to one head; 16-byte copies and loads
+    REQUIRE((K / heads) % vec_elems(dta) == 0 && heads <= 64, SPK_ERR_UNSUPPORTED,
+            "spk_spmm_t_pair: no kernel for K = %d in %d heads", K, heads);
+    REQUIRE(aligned16(A) && aligned16(Y) && aligned16(X) && (lda * dt_bytes(dta)) % 16 == 0 && ldy % 4 == 0 &&
+                ldx % 4 == 0 && (reinterpret_cast<uintptr_t>(cw) & 7u) == 0,
+            SPK_ERR_UNSUPPORTED, "spk_spmm_t_pair: A, Y, X must be 16-byte aligned with 16-byte row strides");
+    const size_t need = (size_t)T.npieces * (size_t)K * 4;
+    if (need > 0) {
+        REQUIRE(workspace && ws_bytes >= need, SPK_ERR_WORKSPACE, "spk_spmm_t_pair: workspace has %zu bytes, needs %zu",
+                workspace ? ws_bytes : (size_t)0, need);
+        REQUIRE(aligned16(workspace), SPK_ERR_WORKSPACE, "spk_spmm_t_pair: workspace must be 16-byte aligned");
+    }
+    if (T.M == 0) return SPK_OK;
+    PairArgs a;
+    a.K = K; a.heads = heads; a.accumulate = accumulate;
+    a.rowptr = T.rowptr; a.colidx = T.colidx; a.rowidx = T.rowidx; a.perm = P->perm; a.cw = cw;
+    a.A = A; a.lda = lda; a.Y = Y; a.ldy = ldy; a.X = X; a.ldx = ldx;
+    a.bnd = T.bnd; a.meta = T.meta; a.head_s0 = T.head_s0; a.slot_np = T.slot_np; a.cnt = T.cnt;
+    a.carry = reinterpret_cast<float*>(workspace);
+    a.nchunks = T.nchunks;
+    cudaError_t e = launch_pair(dta, a, (cudaStream_t)stream);
+    if (e != cudaSuccess) return cuda_fail(e, "spk_spmm_t_pair");
+    return SPK_OK;
 }
 
 // ----------------------------------------------------------------------------

@@ -338,6 +338,8 @@ struct FusedArgs {
     float* Y; int64_t ldy;
     float* scores;            // heads x nnz (head-major), or NULL
     float* lse;               // M x heads: max + log(sum) of each softmax row, or NULL
+    const float* rowdot;      // backward: M x heads, <dY_i, Y_i> of each head
+    float* cw;                // backward: per entry and head its score gradient c and weight w
     const int2* bnd;
     const int4* meta;
     const int32_t* head_s0;
@@ -431,7 +433,7 @@ cudaError_t build_transpose(const int32_t* rowptr, const int32_t* colidx, int64_
                             char* storage, char* temp, const TplanLayout& L, cudaStream_t s);
 // Stable LSD radix sort of n int32 keys (8 bits per pass, `passes` passes over
 // the low bits) carrying int32 values (NULL = the identity 0..n-1); the result
-// lands in k0/v0 or k1/v1 (pointers returned; keys/vals themselves when n = 0
+// lands in k0/v0 or k1/v1, (pointers returned; keys/vals themselves when n = 0
 // or passes = 0).  hist: radix_hist_bytes(n); scan_tmp: scan_temp_bytes of the
 // histogram's entries (radix_tiles(n) * 256).
 int radix_passes(int64_t range);          // passes that cover keys in [0, range)

@@ -288,6 +288,58 @@ def fused_score_grad(S: CSR, w: torch.Tensor, dw: torch.Tensor, rowdot, heads: i
     return de
 
 
+def fused_grad(S: CSR, B: torch.Tensor, dY: torch.Tensor, scores: torch.Tensor, lse, rowdot, heads: int, softmax: bool,
+               scale: float, vals=None) -> tuple[torch.Tensor, torch.Tensor]:
+    """Row side of the FusedMM backward in one pass over S: (dA, cw), dA = M x K
+    FP32, cw = nnz x heads x 2 pairs of the gradient c w.r.t. the unscaled dot
+    <A_i, B_j> and the weight w.  Raises SpkError (SPK_ERR_UNSUPPORTED) where no
+    kernel covers the shape or its alignment."""
+    dtb, ldb = _dense(B, "B", S.device)
+    dtd, lddy = _dense(dY, "dY", S.device)
+    if B.size(0) != S.N or dY.shape != (S.M, B.size(1)) or dtd != SPK_F32:
+        raise ValueError("B must be N x K and dY M x K float32")
+    K = B.size(1)
+    scores = _f32(scores, (heads, S.nnz), "scores", S.device)
+    lse = _f32(lse, (S.M, heads), "lse", S.device) if softmax else None
+    rowdot = _f32(rowdot, (S.M, heads), "rowdot", S.device) if softmax else None
+    vals = _vals(vals, S, "vals")
+    dA = torch.empty((S.M, K), dtype=torch.float32, device=S.device)
+    cw = torch.empty((S.nnz, heads, 2), dtype=torch.float32, device=S.device)
+    ws = S.fused_workspace(K, heads)
+    check(lib().spk_fused_grad(S.handle, scores.data_ptr(), _ptr(lse), _ptr(rowdot), _ptr(vals), float(scale),
+                               int(bool(softmax)), dtb, B.data_ptr(), ldb, dY.data_ptr(), lddy, K, int(heads),
+                               dA.data_ptr(), K, cw.data_ptr(), _ptr(ws), 0 if ws is None else ws.numel(),
+                               _stream(S.device)), "spk_fused_grad")
+    return dA, cw
+
+
+def spmm_t_pair(S: CSR, cw: torch.Tensor, A: torch.Tensor, Y: torch.Tensor, *, out: torch.Tensor | None = None,
+                accumulate: bool = False, plan: TransposePlan | None = None) -> torch.Tensor:
+    """X (+)= S_c^T A + S_w^T Y with the pairs (c, w) of ``fused_grad`` (nnz x
+    heads x 2), through the transpose plan.  FP32 output; Y FP32."""
+    P = plan or S.transpose_plan()
+    dta, lda = _dense(A, "A", S.device)
+    dty, ldy = _dense(Y, "Y", S.device)
+    if dty != SPK_F32 or A.shape != Y.shape or A.size(0) != S.M:
+        raise ValueError("A must be M x K and Y M x K float32")
+    K = A.size(1)
+    if cw.dim() != 3 or cw.dtype != torch.float32 or cw.device != S.device or cw.size(0) != S.nnz or cw.size(2) != 2 \
+            or not cw.is_contiguous():
+        raise ValueError("cw must be float32, nnz x heads x 2, contiguous, on the pattern's device")
+    if out is None:
+        if accumulate:
+            raise ValueError("accumulate needs an output tensor")
+        out = torch.empty((S.N, K), dtype=torch.float32, device=S.device)
+    _, ldx = _dense(out, "out", S.device)
+    if out.dtype != torch.float32 or out.shape != (S.N, K):
+        raise ValueError("out must be N x K float32")
+    ws = P.workspace(K)
+    check(lib().spk_spmm_t_pair(P.handle, cw.data_ptr(), cw.size(1), dta, A.data_ptr(), lda, Y.data_ptr(), ldy, K,
+                                out.data_ptr(), ldx, int(accumulate), _ptr(ws), 0 if ws is None else ws.numel(),
+                                _stream(S.device)), "spk_spmm_t_pair")
+    return out
+
+
 def cast(x: torch.Tensor, dtype) -> torch.Tensor:
     """Round-to-nearest-even cast of an FP32 tensor to bfloat16 / float16."""
     if x.dtype != torch.float32 or not x.is_cuda:
