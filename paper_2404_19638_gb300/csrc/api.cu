@@ -1137,7 +1137,7 @@ extern "C" spk_status spk_tplan_build(spk_csr S, int32_t chunk_work, void* stora
             SPK_ERR_WORKSPACE, "spk_tplan_build: buffers must be 256-byte aligned");
     cudaStream_t s = (cudaStream_t)stream;
     char* st = reinterpret_cast<char*>(storage);
-    cudaError_t e = build_transpose(S->rowptr, S->colidx, S->M, S->N, S->nnz, st, reinterpret_cast<char*>(temp), L, s);
+    cudaError_t e = build_transpose(S->rowptr, S->colidx, S->has_sched ? S->rowidx : nullptr, S->M, S->N, S->nnz, st, reinterpret_cast<char*>(temp), L, s);
     if (e != cudaSuccess) return cuda_fail(e, "spk_tplan_build");
     spk_tplan_s* P = new (std::nothrow) spk_tplan_s();
     REQUIRE(P, SPK_ERR_ARG, "spk_tplan_build: out of host memory");

@@ -429,11 +429,12 @@ cudaError_t launch_fused_score_grad(const int32_t* rowidx, int64_t nnz, int head
 int fused_shape_index(int G, int NV, int U);   // -1 if not compiled
 cudaError_t launch_permute_vals(const int32_t* perm, const float* vals, const float* vals2, int64_t nnz, float* out,
                                 cudaStream_t s);
-cudaError_t build_transpose(const int32_t* rowptr, const int32_t* colidx, int64_t M, int64_t N, int64_t nnz,
-                            char* storage, char* temp, const TplanLayout& L, cudaStream_t s);
+// coo_rows: the schedule's row of every entry, or NULL.
+cudaError_t build_transpose(const int32_t* rowptr, const int32_t* colidx, const int32_t* coo_rows, int64_t M,
+                            int64_t N, int64_t nnz, char* storage, char* temp, const TplanLayout& L, cudaStream_t s);
 // Stable LSD radix sort of n int32 keys (8 bits per pass, `passes` passes over
 // the low bits) carrying int32 values (NULL = the identity 0..n-1); the result
-// lands in k0/v0 or k1/v1, (pointers returned; keys/vals themselves when n = 0
+// lands in k0/v0 or k1/v1, or the last pass in k_last/v_last if given (pointers returned; keys/vals themselves when n = 0
 // or passes = 0).  hist: radix_hist_bytes(n); scan_tmp: scan_temp_bytes of the
 // histogram's entries (radix_tiles(n) * 256).
 int radix_passes(int64_t range);          // passes that cover keys in [0, range)
@@ -441,7 +442,8 @@ int64_t radix_tiles(int64_t n);
 size_t radix_hist_bytes(int64_t n);
 cudaError_t radix_sort_i32(const int32_t* keys, const int32_t* vals, int64_t n, int passes, int32_t* k0, int32_t* k1,
                            int32_t* v0, int32_t* v1, int32_t* hist, void* scan_tmp, const int32_t** keys_out,
-                           const int32_t** vals_out, cudaStream_t s);
+                           const int32_t** vals_out, cudaStream_t s, int32_t* k_last = nullptr,
+                           int32_t* v_last = nullptr);
 // Row relabelling (reorder.cu)
 size_t reorder_temp_bytes(int64_t M);
 cudaError_t row_order(const int32_t* rowptr, const int32_t* colidx, int64_t M, int64_t N, int64_t nnz, int kind,

@@ -163,21 +163,23 @@ cudaError_t coo_to_csr(int64_t M, int64_t N, int64_t nnz, const int32_t* rows, c
         int32_t* v0 = at(L.v0); int32_t* v1 = at(L.v1);
         if (p1 == v0) { v0 = at(L.flag); k0 = at(L.pos); }          // keep p1 intact while it is read
         else if (p1 == v1) { v1 = at(L.flag); k1 = at(L.pos); }
-        e = radix_sort_i32(at(L.keys2), p1, nnz, radix_passes(M), k0, k1, v0, v1, at(L.hist), temp + L.scan, &rs, &p,
-                           s);
-        if (e != cudaSuccess) return e;
-        // copy the final permutation and rows out of the sort buffers that
-        // the flags / positions may reuse
+        // the final permutation and rows go where the flags and positions
+        // do not reuse them
         int32_t* p_fix = at(L.perm);
         int32_t* rs_fix = at(L.rs);
-        if (p) {
+        e = radix_sort_i32(at(L.keys2), p1, nnz, radix_passes(M), k0, k1, v0, v1, at(L.hist), temp + L.scan, &rs, &p,
+                           s, rs_fix, p_fix);
+        if (e != cudaSuccess) return e;
+        if (p && p != p_fix) {                                       // M <= 1: no pass ran
             e = cudaMemcpyAsync(p_fix, p, (size_t)nnz * 4, cudaMemcpyDeviceToDevice, s);
             if (e != cudaSuccess) return e;
             p = p_fix;
         }
-        e = cudaMemcpyAsync(rs_fix, rs, (size_t)nnz * 4, cudaMemcpyDeviceToDevice, s);
-        if (e != cudaSuccess) return e;
-        rs = rs_fix;
+        if (rs != rs_fix) {
+            e = cudaMemcpyAsync(rs_fix, rs, (size_t)nnz * 4, cudaMemcpyDeviceToDevice, s);
+            if (e != cudaSuccess) return e;
+            rs = rs_fix;
+        }
         int32_t* cs = at(L.k0);
         int32_t* flag = dedup ? at(L.flag) : nullptr;
         k_coo_gather<<<grid_for(nnz), 256, 0, s>>>(rs, cols, p, nnz, cs, flag);
