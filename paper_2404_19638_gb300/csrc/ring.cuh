@@ -50,6 +50,14 @@ __device__ __forceinline__ void cpa16_if(bool p, unsigned smem, const void* gmem
                  : "memory");
 }
 
+// CB (4 or 8) bytes from gmem if p, else zeros (gmem is not read).
+template <int CB, int SO = 0>
+__device__ __forceinline__ void cpa_part(bool p, unsigned smem, const void* gmem)
+{
+    asm volatile("cp.async.ca.shared.global [%0+%3], [%1], %4, %2;\n" ::"r"(smem), "l"(gmem), "r"(p ? CB : 0), "n"(SO), "n"(CB)
+                 : "memory");
+}
+
 // for_const<N>(f): f(integral constant 0), ..., f(integral constant N - 1).
 template <int I>
 struct IntC { static constexpr int value = I; __device__ constexpr operator int() const { return I; } };

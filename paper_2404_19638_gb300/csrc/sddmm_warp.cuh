@@ -19,6 +19,11 @@
 // order of each dot (even and odd elements apart, vectors in order, then the
 // reduce-scatter over the lanes) is that of the register path, bit for bit.
 //
+// Rows that 16 bytes do not divide (CB < 16): a lane copies its vectors 8 or 4
+// bytes at a time, zeros past the end of a row; the dots are the same.
+// The element path, 4 bytes a lane into registers: 210 us against 129 (120,011 x
+// 75,503, 20 nonzeros a row, FP32, K = 50).
+//
 // What bounds it (GB300): FP32 rows the shared-memory data path (64-78 %
 // busy) and the latency of the gathers at the 18 warps an SM has room for;
 // 16-bit rows that latency and the issue of one mixed-precision FMA per
@@ -51,6 +56,16 @@ __device__ __forceinline__ ulonglong2 lds16(unsigned smem)
 __device__ __forceinline__ uint4 words(const ulonglong2 v)
 {
     return make_uint4((uint32_t)v.x, (uint32_t)(v.x >> 32), (uint32_t)v.y, (uint32_t)(v.y >> 32));
+}
+
+// The first n of 16 bytes at p, CB bytes a load, zeros after them.
+template <int CB>
+__device__ __forceinline__ ulonglong2 ldg_part(const char* p, int n)
+{
+    uint32_t w[4];
+#pragma unroll
+    for (int c = 0; c < 16; c += 4) w[c / 4] = c / CB * CB < n ? __ldg(reinterpret_cast<const unsigned int*>(p + c)) : 0u;
+    return make_ulonglong2(pack2(w[0], w[1]), pack2(w[2], w[3]));
 }
 
 template <>
@@ -176,8 +191,9 @@ __host__ __device__ constexpr int sddmm_warp_bytes(int G, int NV, int U)      //
 // The chunk's nonzeros [e0, e0 + n).  ALLV: every lane's NV vectors lie inside
 // K.  NH > 0: several heads, each a block of NH consecutive vectors of a row
 // (lane gl's vector t belongs to head (t * G + gl) / NH), one output array of
-// nnz values per head; NH = 0: one dot per nonzero.
-template <int DTA, int DTB, int G, int NV, int U, bool ALLV, int NH = 0>
+// nnz values per head; NH = 0: one dot per nonzero.  CB: bytes of a copy
+// (below 16, ALLV is false).
+template <int DTA, int DTB, int G, int NV, int U, bool ALLV, int NH = 0, int CB = 16>
 __device__ __forceinline__ void sddmm_warp_chunk(const SddmmArgs& a, unsigned char* wsm, int e0, int n)
 {
     using W = SddmmWarp<DTA, DTB, G, NV, U>;
@@ -186,7 +202,8 @@ __device__ __forceinline__ void sddmm_warp_chunk(const SddmmArgs& a, unsigned ch
     constexpr unsigned WMASK = WB == 32 ? 0xffffffffu : (1u << (WB % 32)) - 1u;
     if (n <= 0) return;
     const int lane = threadIdx.x & 31, grp = lane / G, gl = lane % G;
-    const int nvec = a.K / vec_elems(DTB);
+    const int nvec = (a.K + vec_elems(DTB) - 1) / vec_elems(DTB);
+    const int rowA = a.K * dt_bytes(DTA), rowB = a.K * dt_bytes(DTB);
     bool vin[NV];
 #pragma unroll
     for (int t = 0; t < NV; ++t) vin[t] = ALLV || t * G + gl < nvec;
@@ -250,7 +267,17 @@ __device__ __forceinline__ void sddmm_warp_chunk(const SddmmArgs& a, unsigned ch
                 j[4 * c] = v.x; j[4 * c + 1] = v.y; j[4 * c + 2] = v.z; j[4 * c + 3] = v.w;
             }
             const bool whole = ALLV && left >= WB;
-            if (whole) {
+            if constexpr (CB < 16) {
+                for_const<U>([&](auto u) {
+                    const bool on = grp * U + u.value < left;
+                    const char* p = Bb + (on ? (size_t)(unsigned)j[u.value] * ldb_bytes : 0);
+                    for_const<NV * (16 / CB)>([&](auto q) {
+                        constexpr int t = q.value / (16 / CB), o = t * G * 16 + q.value % (16 / CB) * CB;
+                        const bool in = on && gl * 16 + o < rowB;
+                        cpa_part<CB, SB + (u.value * NV + t) * 512 + q.value % (16 / CB) * CB>(in, smB, in ? p + o : Bb);
+                    });
+                });
+            } else if (whole) {
                 for_const<U>([&](auto u) {
                     const char* p = Bb + (size_t)(unsigned)j[u.value] * ldb_bytes;
                     for_const<NV>([&](auto t) {
@@ -272,6 +299,14 @@ __device__ __forceinline__ void sddmm_warp_chunk(const SddmmArgs& a, unsigned ch
                 const bool mine = grp < NA - 1 ? grp < cnt : cnt >= NA;
                 const int r = mine ? arow[o / WB * NA + grp] : 0;
                 const char* p = Ab + (size_t)(unsigned)r * lda_bytes;
+                if constexpr (CB < 16)
+                    for_const<NV * VA * (16 / CB)>([&](auto q) {
+                        constexpr int v = q.value / (16 / CB), c = q.value % (16 / CB) * CB;
+                        constexpr int o = v / VA * G * 16 * VA + v % VA * 16 + c;
+                        const bool in = mine && gl * 16 * VA + o < rowA;
+                        cpa_part<CB, SA + v * 512 + c>(in, smA, in ? p + o : Ab);
+                    });
+                else
                 for_const<NV * VA>([&](auto q) {
                     constexpr int t = q.value / VA, h = q.value % VA;
                     cpa16_if<SA + q.value * 512, t * G * 16 * VA + h * 16>(mine && vin[t], smA, p);
@@ -332,8 +367,11 @@ __device__ __forceinline__ void sddmm_warp_chunk(const SddmmArgs& a, unsigned ch
                             for (int t = 0; t < NV; ++t)
                                 if (vin[t])
 #pragma unroll
-                                    for (int h = 0; h < VA; ++h)
-                                        av[t].set(h, __ldg(reinterpret_cast<const ulonglong2*>(q + t * G * 16 * VA + h * 16)));
+                                    for (int h = 0; h < VA; ++h) {
+                                        const char* x = q + t * G * 16 * VA + h * 16;
+                                        if constexpr (CB < 16) av[t].set(h, ldg_part<CB>(x, rowA - (gl * 16 * VA + t * G * 16 * VA + h * 16)));
+                                        else av[t].set(h, __ldg(reinterpret_cast<const ulonglong2*>(x)));
+                                    }
                         }
                     }
                     turn = false;
@@ -417,6 +455,14 @@ __device__ __forceinline__ void sddmm_warp_chunk(const SddmmArgs& a, unsigned ch
 }
 
 // One warp per CTA and chunk, so that every per-chunk quantity is uniform.
+template <int DTA, int DTB, int G, int NV, int U, int CB>
+__global__ void __launch_bounds__(32) k_sddmm_warp_part(const SddmmArgs a)
+{
+    extern __shared__ __align__(16) unsigned char ring_smem[];
+    const int e0 = a.bnd[blockIdx.x].y;
+    sddmm_warp_chunk<DTA, DTB, G, NV, U, false, 0, CB>(a, ring_smem, e0, a.bnd[blockIdx.x + 1].y - e0);
+}
+
 template <int DTA, int DTB, int G, int NV, int U>
 __global__ void __launch_bounds__(32) k_sddmm_warp(const SddmmArgs a)
 {
@@ -438,6 +484,31 @@ cudaError_t launch_sddmm_warp_shape(const SddmmArgs& a, cudaStream_t s)
     }
     void* args[] = {(void*)&a};
     return cudaLaunchKernel(fn, dim3((unsigned)a.nchunks), dim3(32), args, smem, s);
+}
+
+// Rows of nv vectors (the last one partial), copied CB bytes at a time.
+template <int DTA, int DTB, int G, int NV, int U, int CB>
+cudaError_t launch_sddmm_part_shape(const SddmmArgs& a, cudaStream_t s)
+{
+    const void* fn = (const void*)&k_sddmm_warp_part<DTA, DTB, G, NV, U, CB>;
+    constexpr int smem = SddmmWarp<DTA, DTB, G, NV, U>::BYTES;
+    if (smem > 48 * 1024) {
+        cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        if (e != cudaSuccess) return e;
+    }
+    void* args[] = {(void*)&a};
+    return cudaLaunchKernel(fn, dim3((unsigned)a.nchunks), dim3(32), args, smem, s);
+}
+
+template <int DTA, int DTB, int CB>
+cudaError_t launch_sddmm_part_cb(const SddmmArgs& a, cudaStream_t s)
+{
+    if (a.nchunks <= 0) return cudaSuccess;
+    const int nv = (a.K + vec_elems(DTB) - 1) / vec_elems(DTB);
+    if (nv <= 4) return launch_sddmm_part_shape<DTA, DTB, 4, 1, 4, CB>(a, s);
+    if (nv <= 8) return launch_sddmm_part_shape<DTA, DTB, 4, 2, 4, CB>(a, s);
+    if (nv <= 16) return launch_sddmm_part_shape<DTA, DTB, 8, 2, 4, CB>(a, s);
+    return launch_sddmm_part_shape<DTA, DTB, 8, 4, 4, CB>(a, s);
 }
 
 }  // namespace spk

@@ -25,6 +25,12 @@
 // Every output element adds its nonzeros in slot order with one FMA each, as
 // the row-split and register paths do, so all paths agree bit for bit.
 //
+// Rows that 16 bytes do not divide (CB < 16) are copied 8 or 4 bytes at a
+// time, one per lane, and written element by element; the rest is the same.
+// The element path reads each row 4 bytes a lane into registers, one lane
+// group a chunk: 171 us against 118 (120,011 x 75,503, 20 nonzeros a
+// row, FP32, K = 50).
+//
 // What bounds it (GB300, R-MAT scale 20, 16.1M nonzeros, K = 64): the
 // shared-memory data path, 75 % busy in FP32 (each gathered row is written and
 // read once there), and instruction issue for 16-bit rows (the widening).
@@ -126,9 +132,18 @@ __device__ __forceinline__ void write_vec_at(const SpmmArgs& a, char* p, const f
     write_vec<E>(b, 0, v);
 }
 
+// The first ne elements of a lane's part of an output row, one by one.
+template <int E>
+__device__ __forceinline__ void write_some_at(const SpmmArgs& a, char* p, const float* v, int ne, int celt)
+{
+#pragma unroll
+    for (int q = 0; q < E; ++q)
+        if (q < ne) write_vec_at<1>(a, p + q * celt, v + q);
+}
+
 // A piece of a split row is in its carry slot: the warp that delivers the last
 // one adds the pieces in slot order and writes the row.
-template <int DT, int CL>
+template <int DT, int CL, int CB>
 __device__ __noinline__ void spmm_warp_finish(const SpmmArgs& a, int nkb, int s0, int64_t row)
 {
     using W = SpmmWarp<DT, CL>;
@@ -148,17 +163,28 @@ __device__ __noinline__ void spmm_warp_finish(const SpmmArgs& a, int nkb, int s0
     for (int kb = 0; kb < nkb; ++kb) {
         const int c = kb * (W::RBB / dt_bytes(DT)) + lane * E;
         if (lane * W::LB < min(a.K * dt_bytes(DT) - kb * W::RBB, W::RBB)) {
+            const int ne = CB < 16 ? min(E, a.K - c) : E;
             float sum[E];
 #pragma unroll
             for (int q = 0; q < E; ++q) sum[q] = 0.f;
 #pragma unroll 4
             for (int sl = s0; sl < s0 + np; ++sl) {
                 float x[E];
-                load_elems_cg<DT_F32, E>(a.carry, (int64_t)sl * a.K + c, x);
+                if constexpr (CB < 16) {
+#pragma unroll
+                    for (int q = 0; q < E; ++q) x[q] = q < ne ? __ldcg(a.carry + (int64_t)sl * a.K + c + q) : 0.f;
+                } else {
+                    load_elems_cg<DT_F32, E>(a.carry, (int64_t)sl * a.K + c, x);
+                }
 #pragma unroll
                 for (int q = 0; q < E; ++q) sum[q] += x[q];
             }
-            write_vec<E>(a, row * a.ldc + c, sum);
+            if constexpr (CB < 16) {
+                const int celt = dt_bytes_rt(a.dtc);
+                write_some_at<E>(a, reinterpret_cast<char*>(a.C) + (row * a.ldc + c) * celt, sum, ne, celt);
+            } else {
+                write_vec<E>(a, row * a.ldc + c, sum);
+            }
         }
     }
     __syncwarp();
@@ -166,7 +192,8 @@ __device__ __noinline__ void spmm_warp_finish(const SpmmArgs& a, int nkb, int s0
 }
 
 // FULL: every K block is CL * 16 bytes wide, so every lane copies and accumulates.
-template <int DT, int CL, int MODE, bool FULL>
+// CB: bytes of a copy; below 16, MODE is SPMM_ANY and FULL false.
+template <int DT, int CL, int MODE, bool FULL, int CB = 16>
 __device__ __forceinline__ void spmm_warp_span(const SpmmArgs& a, unsigned char* wsm, int kb, int nkb, const int2 b0,
                                                const int2 b1, const int4 meta, int head_s0)
 {
@@ -232,8 +259,22 @@ __device__ __forceinline__ void spmm_warp_span(const SpmmArgs& a, unsigned char*
     // their columns)
     constexpr bool BLK = NS % 4 == 0;
     const unsigned slot0 = (unsigned)__cvta_generic_to_shared(wsm) + (BLK ? sub * NS : sub) * W::RBB + vec * 16;
+    static_assert(CB == 16 || (MODE == SPMM_ANY && !FULL), "");
+    const int ne = CB < 16 ? min(E, rb / dt_bytes(DT) - lane * E) : E;      // columns of this lane
     auto issue = [&](const int* cols, unsigned slot, int left) {    // copy a batch of `left` (or U) rows
-        if (left > 0) {
+        if constexpr (CB < 16) {
+            constexpr int VPR = W::RBB / CB;                        // copies of a row
+            const unsigned dst = slot - (BLK ? sub * NS : sub) * W::RBB - vec * 16 + lane * CB;
+            if (left > 0)
+                for_const<U * VPR / 32>([&](auto q) {
+                    const int r = VPR >= 32 ? q.value / (VPR / 32) : (lane + 32 * q.value) / VPR;
+                    const int off = (VPR >= 32 ? lane + 32 * (q.value % (VPR / 32)) : lane % VPR) * CB;
+                    const bool in = off < rb && r < left;
+                    const char* p = reinterpret_cast<const char*>(a.B) + (int64_t)kb * W::RBB;
+                    if (in) p += (size_t)(unsigned)cols[r] * ldb_bytes + off;
+                    cpa_part<CB, q.value * 32 * CB>(in, dst, p);
+                });
+        } else if (left > 0) {
             int j[NS];
             if constexpr (BLK) {
 #pragma unroll
@@ -277,8 +318,18 @@ __device__ __forceinline__ void spmm_warp_span(const SpmmArgs& a, unsigned char*
             float f[E];
             acc.get(f);
             if constexpr (MODE == SPMM_ANY) {
-                if (piece) store_elems<DT_F32, E>(dst, 0, f);
-                else write_vec_at<E>(a, dst, f);
+                if constexpr (CB < 16) {
+                    if (piece) {
+#pragma unroll
+                        for (int q = 0; q < E; ++q)
+                            if (q < ne) reinterpret_cast<float*>(dst)[q] = f[q];
+                    } else {
+                        write_some_at<E>(a, dst, f, ne, celt);
+                    }
+                } else {
+                    if (piece) store_elems<DT_F32, E>(dst, 0, f);
+                    else write_vec_at<E>(a, dst, f);
+                }
             } else {
                 if constexpr (MODE == SPMM_ADD) {
                     if (!piece) {
@@ -350,7 +401,8 @@ __device__ __forceinline__ void spmm_warp_span(const SpmmArgs& a, unsigned char*
                 char* p = Cl + (r0 + __ffs(zm) - 1) * ldc_bytes;
                 zm &= zm - 1;
                 if (!act) continue;
-                if constexpr (MODE == SPMM_ANY) write_vec_at<E>(a, p, z);
+                if constexpr (CB < 16) write_some_at<E>(a, p, z, ne, celt);
+                else if constexpr (MODE == SPMM_ANY) write_vec_at<E>(a, p, z);
                 else store_elems<DT_F32, E>(p, 0, z);
             }
         }
@@ -395,14 +447,14 @@ __device__ __forceinline__ void spmm_warp_span(const SpmmArgs& a, unsigned char*
         dst = carry_slot(meta.y);
     }
     close();
-    if (meta.x >= 0) spmm_warp_finish<DT, CL>(a, nkb, head_s0, b0.x);
-    if (meta.y >= 0) spmm_warp_finish<DT, CL>(a, nkb, meta.y, b1.x);
+    if (meta.x >= 0) spmm_warp_finish<DT, CL, CB>(a, nkb, head_s0, b0.x);
+    if (meta.y >= 0) spmm_warp_finish<DT, CL, CB>(a, nkb, meta.y, b1.x);
 }
 
 // One warp per CTA and chunk (so that every per-chunk quantity is uniform over
 // the CTA and row changes are plain branches), one grid row per K block of
 // CL * 16 bytes.
-template <int DT, int CL, int MODE, bool FULL>
+template <int DT, int CL, int MODE, bool FULL, int CB = 16>
 __global__ void __launch_bounds__(32) k_spmm_warp(const SpmmArgs a)
 {
     extern __shared__ __align__(16) unsigned char ring_smem[];
@@ -410,16 +462,22 @@ __global__ void __launch_bounds__(32) k_spmm_warp(const SpmmArgs a)
     const int2 b0 = a.bnd[c], b1 = a.bnd[c + 1];
     const int4 m = a.meta[c];
     const int hs0 = (m.x >= 0) ? __ldg(a.head_s0 + c) : -1;
-    spmm_warp_span<DT, CL, MODE, FULL>(a, ring_smem, blockIdx.y, gridDim.y, b0, b1, m, hs0);
+    spmm_warp_span<DT, CL, MODE, FULL, CB>(a, ring_smem, blockIdx.y, gridDim.y, b0, b1, m, hs0);
 }
 
-template <int DT, int CL>
+template <int DT, int CL, int CB = 16>
 cudaError_t launch_spmm_warp_cl(const SpmmArgs& a, cudaStream_t s)
 {
     using W = SpmmWarp<DT, CL>;
     const int rb = a.K * dt_bytes(DT);
     const int nkb = (rb + W::RBB - 1) / W::RBB;
     if (nkb > 65535) return cudaErrorInvalidValue;
+    if constexpr (CB < 16) {
+        const void* fn = (const void*)&k_spmm_warp<DT, CL, SPMM_ANY, false, CB>;
+        const size_t smem = W::bytes(a.heads);
+        void* args[] = {(void*)&a};
+        return cudaLaunchKernel(fn, dim3((unsigned)a.nchunks, (unsigned)nkb), dim3(32), args, smem, s);
+    } else {
     const int mode = a.dtc != DT_F32 ? SPMM_ANY : (a.accumulate ? SPMM_ADD : SPMM_STORE);
     const bool full = rb % W::RBB == 0;
     const void* fn = mode == SPMM_STORE ? (full ? (const void*)&k_spmm_warp<DT, CL, SPMM_STORE, true>
@@ -435,20 +493,21 @@ cudaError_t launch_spmm_warp_cl(const SpmmArgs& a, cudaStream_t s)
     }
     void* args[] = {(void*)&a};
     return cudaLaunchKernel(fn, dim3((unsigned)a.nchunks, (unsigned)nkb), dim3(32), args, smem, s);
+    }
 }
 
 // K blocks of the smallest 2^k x 32 bytes that holds a row, at most 512.
-template <int DT>
+template <int DT, int CB = 16>
 cudaError_t launch_spmm_warp(SpmmArgs a, cudaStream_t s)
 {
     if (a.nchunks <= 0) return cudaSuccess;
     if (!a.vals) a.heads = 1;                            // ones for every head
     const int rb = a.K * dt_bytes(DT);
-    if (rb <= 32) return launch_spmm_warp_cl<DT, 2>(a, s);
-    if (rb <= 64) return launch_spmm_warp_cl<DT, 4>(a, s);
-    if (rb <= 128) return launch_spmm_warp_cl<DT, 8>(a, s);
-    if (rb <= 256) return launch_spmm_warp_cl<DT, 16>(a, s);
-    return launch_spmm_warp_cl<DT, 32>(a, s);
+    if (rb <= 32) return launch_spmm_warp_cl<DT, 2, CB>(a, s);
+    if (rb <= 64) return launch_spmm_warp_cl<DT, 4, CB>(a, s);
+    if (rb <= 128) return launch_spmm_warp_cl<DT, 8, CB>(a, s);
+    if (rb <= 256) return launch_spmm_warp_cl<DT, 16, CB>(a, s);
+    return launch_spmm_warp_cl<DT, 32, CB>(a, s);
 }
 
 }  // namespace spk
