@@ -83,7 +83,8 @@ def peaks():
 # The files the step kernels (k_sddmm_ring, k_spmm_ring and their register
 # and row-split siblings) compile from: a change elsewhere in csrc/ (FusedMM,
 # batch, tensor-core tiles, plans) leaves their ncu traffic valid.
-STEP_KERNEL_SOURCES = ("common.cuh", "tiles.cuh", "lean.cuh", "ring.cuh", "sddmm_impl.cuh", "spmm_impl.cuh",
+STEP_KERNEL_SOURCES = ("common.cuh", "tiles.cuh", "lean.cuh", "ring.cuh", "rows.cuh", "sddmm_impl.cuh", "spmm_impl.cuh",
+                       "sddmm_warp.cuh", "spmm_warp.cuh",
                        "sddmm_f32.cu", "sddmm_bf16.cu", "sddmm_f16.cu", "sddmm_e4m3.cu",
                        "spmm_f32.cu", "spmm_bf16.cu", "spmm_f16.cu", "spmm_e4m3.cu")
 

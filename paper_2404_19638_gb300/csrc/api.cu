@@ -685,34 +685,28 @@ extern "C" spk_status spk_fusedmm(spk_csr S, const float* vals, float scale, int
     REQUIRE(!vals || aligned16(vals), SPK_ERR_ARG, "spk_fusedmm: vals must be 16-byte aligned");
     const int nvh = dh / vecn;
     const int nv = K / vecn;
-    // Kernel choice.  The all-heads kernel (one lane group per row, heads as
-    // blocks of G / heads lanes, NV adjacent vectors a lane) when a row is at
-    // most 32 vectors and the heads split the lanes evenly; else, or when a
-    // shape is asked for, the one-head-per-grid-row kernel.  Measured on
-    // rmat20, K = 64, GB300: one head runs best on the one-head kernel (FP32
-    // 8 lanes x 2 vectors 0.85 ms, 16-bit 8 lanes 0.86 ms, against 1.16 / 1.24
-    // on the all-heads kernel); 16-bit rows with 4 or more heads on the
-    // all-heads kernel with 2 vectors a lane (1.21 ms against 1.32).
-    // tune.vecs_per_lane alone (no group_lanes, no unroll) asks for the
-    // all-heads kernel with that many vectors a lane (1 or 2).
+    // Kernel choice: the warp kernel for all heads (fused_warp.cuh) wherever it
+    // covers the call, i.e. rows of at most 512 bytes and one head or heads of
+    // a power of two 16-byte vectors.  It was the faster one at every width,
+    // head count and dtype measured (R-MAT of 8M nonzeros and 5 nonzeros a row,
+    // K = 16-128, 1-4 heads; narrowest margin FP32 K = 128 in 4 heads at 5 a
+    // row: 0.277 against 0.313 ms).  Wider rows and other heads run one head per
+    // grid row, and so does a shape that is asked for; tune.vecs_per_lane alone
+    // (no group_lanes, no unroll) asks for the lane-group kernel of all heads
+    // with that many vectors a lane (1 or 2).
     const bool mh_asked = tune && tune->vecs_per_lane && !tune->group_lanes && !tune->unroll;
-    const bool shaped = tune && (tune->group_lanes || tune->unroll || (tune->vecs_per_lane && !mh_asked));
+    const bool shaped = tune && (tune->group_lanes || tune->unroll);
     const bool one_head = heads == 1 && ((dt == SPK_F32 && nvh == 16) || (dt != SPK_F32 && nvh == 8));
-    auto mh_fits = [&](int nvl) {
-        const int g = nv / nvl;
-        return nv % nvl == 0 && (g == 4 || g == 8 || g == 16 || (g == 32 && nvl == 1)) && g % heads == 0;
-    };
-    int mh_nv = 1;
+    const int mh_nv = mh_asked ? tune->vecs_per_lane : 1;
     if (mh_asked) {
-        mh_nv = tune->vecs_per_lane;
         REQUIRE(mh_nv == 1 || mh_nv == 2, SPK_ERR_ARG, "spk_fusedmm: vecs_per_lane must be 1 or 2 for the all-heads kernel");
-        REQUIRE(mh_fits(mh_nv), SPK_ERR_UNSUPPORTED,
-                "spk_fusedmm: %d vectors a row do not split into %d heads of %d-vector lanes", nv, heads, mh_nv);
-    } else if (dt != SPK_F32 && heads >= 4 && mh_fits(2)) {
-        mh_nv = 2;
+        const int g = nv / mh_nv;
+        REQUIRE(nv % mh_nv == 0 && (g == 4 || g == 8 || g == 16 || (g == 32 && mh_nv == 1)) && g % heads == 0,
+                SPK_ERR_UNSUPPORTED, "spk_fusedmm: %d vectors a row do not split into %d heads of %d-vector lanes", nv,
+                heads, mh_nv);
     }
     const bool warp = !shaped && !mh_asked && fused_warp_supported(dt, K, heads);
-    const bool mh = mh_asked || (!shaped && !one_head && mh_fits(mh_nv));
+    const bool mh = mh_asked;
     int G, NV = 1, U = 4, idx = -1;
     if (!mh && !warp) {
         if (nvh <= 4) G = 4;

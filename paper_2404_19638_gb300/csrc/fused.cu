@@ -7,8 +7,12 @@
 // head instead of two, and the scores never travel through HBM (they are
 // written only if asked for).
 //
-// Structure: the SpMM ring span (ring.cuh) with one lane group per span of the
-// balanced schedule and one head per grid row (blockIdx.y); a group covers a
+// These kernels run rows of more than 512 bytes, heads that are not a power of
+// two of 16-byte vectors, and shapes that are asked for; all other calls run
+// fused_warp.cuh.
+//
+// Structure: a span of the balanced schedule per lane group, gathers through a
+// shared-memory ring (ring.cuh) and one head per grid row (blockIdx.y); a group covers a
 // whole head, so each score is complete after a butterfly all-reduce across
 // the group.  The A slice of the current row arrives through the ring when a
 // batch starts a new row.  Row softmax is online: the group keeps the running

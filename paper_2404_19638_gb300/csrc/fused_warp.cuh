@@ -24,11 +24,13 @@
 // batch instead of 4 (R-MAT scale 20, BF16, K = 64, one head: 0.63 ms, this 0.52).
 // Measured against the lane-group kernels of fused.cu, which stay for rows over
 // 512 bytes, heads of other widths and asked-for shapes: R-MAT scale 20,
-// K = 64, softmax: BF16 one head 0.94 -> 0.52 ms, FP32 4 heads with scores and
+// K = 64, softmax: BF16 one head 0.94 -> 0.51 ms, FP32 4 heads with scores and
 // lse 1.26 -> 0.89 ms; R-MAT of 8M nonzeros, K = 16 / 32 / 64 / 128 one head:
-// FP32 0.43 / 0.54 / 0.56 / 0.95 -> 0.29 / 0.30 / 0.38 / 0.63 ms, BF16 0.70 /
-// 0.49 / 0.58 / 0.75 -> 0.23 / 0.29 / 0.29 / 0.43 ms; 5 nonzeros a row, K = 64:
-// 0.24 -> 0.15 and 0.28 -> 0.13 ms.  Bound by instruction issue.
+// FP32 0.43 / 0.54 / 0.56 / 0.95 -> 0.24 / 0.26 / 0.37 / 0.63 ms, BF16 0.70 /
+// 0.49 / 0.58 / 0.75 -> 0.23 / 0.23 / 0.27 / 0.42 ms; 5 nonzeros a row, K = 64:
+// 0.24 -> 0.15 and 0.28 -> 0.11 ms.  Bound by instruction issue (FP32 4 heads:
+// 36 warp instructions per nonzero, issue active in half the cycles at 15 warps
+// an SM, which shared memory limits).
 // Backward (GRAD): A is dY, the dot is dw = <dY_i, B_j>, the weight step makes
 // w (or exp(score - lse)) and c = scale * s * w * (dw - rowdot_i), writes both
 // for S^T, and the add step gives dA_i = sum c B_j: one gather of B for what
@@ -40,10 +42,25 @@
 
 namespace spk {
 
-template <int DTA, int DT, int CL, bool GRAD>
+// Nonzeros per batch.  A batch costs a reduction, a weight step and the loop
+// around them whatever it holds, and its slots cost resident warps; the weight
+// step of one head leaves half the lanes idle at 16.  Measured (R-MAT of 8M
+// nonzeros, softmax, us): forward K = 64 FP32 8 / 16 rows 487 / 376, BF16 8 / 16 /
+// 32 rows 416 / 284 / 274, K = 32 16 / 32 rows FP32 302 / 255, BF16 293 / 233;
+// 32 rows with 2 heads, BF16 K = 64: 316 against 277; 512-byte rows 4 / 8 rows
+// 860 / 626.  Backward, 256-byte rows, 4 heads (its copies of score, lse and
+// row term grow with the batch), R-MAT scale 20: 16 / 8 rows 968 / 823; the
+// graph layer with 128-byte rows 16 / 32 rows 3912 / 3980 a pass.
+constexpr int fused_warp_batch(bool grad, int row_bytes, int heads)
+{
+    if (row_bytes > (grad ? 128 : 256)) return 8;
+    return !grad && heads == 1 && row_bytes <= 128 ? 32 : 16;
+}
+
+template <int DTA, int DT, int CL, bool GRAD, int UB>
 struct FusedWarp {
     static constexpr int RBB = CL * 16;                                       // bytes of a row of B, at most
-    static constexpr int U = RBB > 256 ? 8 : 16;                              // nonzeros per batch
+    static constexpr int U = UB;
     static constexpr int LB = RBB / 32 > dt_bytes(DT) ? RBB / 32 : dt_bytes(DT);  // bytes of a row one lane holds
     static constexpr int E = LB / dt_bytes(DT);
     static constexpr int P = (E + 1) / 2;
@@ -129,13 +146,13 @@ __device__ __noinline__ void fused_warp_finish(const FusedArgs& a, bool smax, in
 }
 
 // FULL: a row of B is CL * 16 bytes.
-template <int DTA, int DT, int CL, bool GRAD, bool FULL>
+template <int DTA, int DT, int CL, bool GRAD, int UB, bool FULL>
 __device__ __forceinline__ void fused_warp_span(const FusedArgs& a, unsigned char* wsm, const int2 b0, const int2 b1,
                                                 const int4 meta, int head_s0)
 {
-    using W = FusedWarp<DTA, DT, CL, GRAD>;
+    using W = FusedWarp<DTA, DT, CL, GRAD, UB>;
     constexpr int E = W::E, P = W::P, U = W::U, NS = W::NS, BPT = W::BPT, NA = W::NA, VA = W::VA;
-    constexpr unsigned UMASK = (1u << U) - 1u;
+    constexpr unsigned UMASK = 0xffffffffu >> (32 - U);
     const int lane = threadIdx.x & 31;
     const int e0 = b0.y, n = b1.y - b0.y;
     const int heads = a.heads;
@@ -530,7 +547,7 @@ __device__ __forceinline__ void fused_warp_span(const FusedArgs& a, unsigned cha
     if (meta.y >= 0) fused_warp_finish<E>(a, !GRAD && smax, head, lead, act, col0, meta.y, b1.x);
 }
 
-template <int DTA, int DT, int CL, bool GRAD, bool FULL>
+template <int DTA, int DT, int CL, bool GRAD, int UB, bool FULL>
 __global__ void __launch_bounds__(32, CL == 8 && DT != DT_F32 ? 24 : 20)
 k_fused_warp(const FusedArgs a)
 {
@@ -539,16 +556,16 @@ k_fused_warp(const FusedArgs a)
     const int2 b0 = a.bnd[c], b1 = a.bnd[c + 1];
     const int4 m = a.meta[c];
     const int hs0 = (m.x >= 0) ? __ldg(a.head_s0 + c) : -1;
-    fused_warp_span<DTA, DT, CL, GRAD, FULL>(a, ring_smem, b0, b1, m, hs0);
+    fused_warp_span<DTA, DT, CL, GRAD, UB, FULL>(a, ring_smem, b0, b1, m, hs0);
 }
 
-template <int DTA, int DT, int CL, bool GRAD>
-cudaError_t launch_fused_warp_cl(const FusedArgs& a, cudaStream_t s)
+template <int DTA, int DT, int CL, bool GRAD, int UB>
+cudaError_t launch_fused_warp_u(const FusedArgs& a, cudaStream_t s)
 {
-    using W = FusedWarp<DTA, DT, CL, GRAD>;
+    using W = FusedWarp<DTA, DT, CL, GRAD, UB>;
     const bool full = a.K * dt_bytes(DT) == W::RBB;
-    const void* fn = full ? (const void*)&k_fused_warp<DTA, DT, CL, GRAD, true>
-                          : (const void*)&k_fused_warp<DTA, DT, CL, GRAD, false>;
+    const void* fn = full ? (const void*)&k_fused_warp<DTA, DT, CL, GRAD, UB, true>
+                          : (const void*)&k_fused_warp<DTA, DT, CL, GRAD, UB, false>;
     const size_t smem = W::bytes(a.heads);
     if (smem > 48 * 1024) {
         cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -556,6 +573,13 @@ cudaError_t launch_fused_warp_cl(const FusedArgs& a, cudaStream_t s)
     }
     void* args[] = {(void*)&a};
     return cudaLaunchKernel(fn, dim3((unsigned)a.nchunks), dim3(32), args, smem, s);
+}
+
+template <int DTA, int DT, int CL, bool GRAD>
+cudaError_t launch_fused_warp_cl(const FusedArgs& a, cudaStream_t s)
+{
+    constexpr int U1 = fused_warp_batch(GRAD, CL * 16, 1), U2 = fused_warp_batch(GRAD, CL * 16, 2);
+    return a.heads == 1 ? launch_fused_warp_u<DTA, DT, CL, GRAD, U1>(a, s) : launch_fused_warp_u<DTA, DT, CL, GRAD, U2>(a, s);
 }
 
 template <int DTA, int DT, bool GRAD>
