@@ -203,7 +203,9 @@ cudaError_t launch_spmm_t(const Launch& L, const SpmmArgs& a, cudaStream_t s)
     const int nkb = (nvec + sh.G * sh.NV - 1) / (sh.G * sh.NV);
     const int64_t items = a.bnd ? a.nchunks : a.M;
     if (items <= 0) return cudaSuccess;
-    if (L.vec && L.ring && a.bnd) return launch_spmm_warp<DTB>(a, s);
+    // The warp kernel has a grid row per 512 bytes of a row of B, and a grid at most 65,535 of them.  Wider rows
+    // (K > 8,388,480 in FP32) take the register path, whose K blocks are up to 2 KB wide.
+    if (L.vec && L.ring && a.bnd && (int64_t)a.K * dt_bytes(DTB) <= SPMM_WARP_MAX_ROW) return launch_spmm_warp<DTB>(a, s);
     const int64_t groups_per_cta = L.threads / sh.G;
     int64_t blocks = (items + groups_per_cta - 1) / groups_per_cta;
     if (blocks > 0x7fffffffLL) blocks = 0x7fffffffLL;

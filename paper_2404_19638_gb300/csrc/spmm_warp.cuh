@@ -51,6 +51,8 @@ namespace spk {
 // dtype and mode decided at run time.
 enum : int { SPMM_STORE = 0, SPMM_ADD = 1, SPMM_ANY = 2 };
 
+constexpr int64_t SPMM_WARP_MAX_ROW = 65535LL * 512;    // bytes of a row: K blocks of 512, one grid row each
+
 template <int DT, int CL>
 struct SpmmWarp {
     static constexpr int RBB = CL * 16;                                       // row bytes of a K block

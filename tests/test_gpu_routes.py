@@ -1,0 +1,30 @@
+"""Which calls reach which kernel: sizes at the limits of the one-warp-per-chunk
+kernels, where another route answers."""
+import numpy as np
+import pytest
+import torch
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda"
+
+
+@pytest.fixture(scope="module")
+def spk():
+    if not torch.cuda.is_available():
+        pytest.skip("needs a CUDA GPU")
+    import paper_2404_19638_gb300 as m
+    return m
+
+
+@pytest.mark.parametrize("K", [65535 * 128, 65535 * 128 + 4])
+def test_spmm_rows_around_the_grid_limit(spk, K):
+    """65,535 K blocks of 512 bytes, and one vector more.  One entry a row: exactly the product."""
+    rp, ci = np.array([0, 1, 1, 2], np.int32), np.array([1, 0], np.int32)
+    v = torch.tensor([0.75, -3.0], device=DEV)
+    S = spk.CSR(rp, ci, (3, 2), v, device=DEV)
+    g = torch.Generator(device=DEV).manual_seed(0)
+    B = torch.randn(2, K, generator=g, device=DEV)
+    C = spk.spmm(S, B)
+    assert torch.equal(C[0], v[0] * B[1]) and torch.equal(C[2], v[1] * B[0]) and not C[1].any()
+    X = spk.spmm_t(S, C)
+    assert torch.equal(X[1], v[0] * C[0]) and torch.equal(X[0], v[1] * C[2])
