@@ -70,13 +70,16 @@ typedef enum spk_dtype {
 typedef struct spk_tune {
     int32_t variant;        /* 0 default, 1 row-split (one lane group per row),
                                2 balanced chunks (merge-path schedule, needs spk_schedule_build),
-                                 gathered rows staged in shared memory where the path supports it,
+                                 one warp per chunk, gathered rows staged in shared memory.  The
+                                 shape fields apply to SDDMM on rows of whole 16-byte vectors and
+                                 where rows are staged in registers; SpMM and rows that 16 bytes
+                                 do not divide have one layout per row width,
                                3 balanced chunks, gathered rows held in registers */
     int32_t group_lanes;    /* lanes that share one row of the dense factor: 4, 8, 16, 32 */
     int32_t vecs_per_lane;  /* 16-byte vectors each lane holds per K block: 1, 2, 4 */
     int32_t unroll;         /* nonzeros in flight per group: 4, 8                  */
     int32_t cta_threads;    /* threads per CTA: 128 or 256 (register paths)        */
-    int32_t stages;         /* batch slots of a shared-memory ring: 2 or 4         */
+    int32_t stages;         /* 2 or 4; accepted, every kernel has two batch slots  */
 } spk_tune;
 
 typedef struct spk_csr_s* spk_csr;       /* pattern of S (+ its schedule)      */
@@ -93,7 +96,8 @@ int32_t spk_version(void);
  * writes min(count, capacity) triples to out (may be NULL), returns count. */
 int32_t spk_shapes(int32_t* out, int32_t capacity);
 /* The tune a default call would use for this op (0 SDDMM, 1 SpMM, 2 SpMM^T),
- * dtype of the gathered operand, and K.  Fills *out. */
+ * dtype of the gathered operand, and K.  Fills *out.  Passed back, it runs the
+ * kernel that a call without a tune runs. */
 spk_status spk_tune_default(spk_csr S, int32_t op, spk_dtype dt, int32_t K, spk_tune* out);
 
 /* ------------------------------------------------------------- pattern -- */

@@ -28,3 +28,22 @@ def test_spmm_rows_around_the_grid_limit(spk, K):
     assert torch.equal(C[0], v[0] * B[1]) and torch.equal(C[2], v[1] * B[0]) and not C[1].any()
     X = spk.spmm_t(S, C)
     assert torch.equal(X[1], v[0] * C[0]) and torch.equal(X[0], v[1] * C[2])
+
+
+@pytest.mark.parametrize("dt,K", [(torch.float32, 18), (torch.float32, 50), (torch.float32, 64), (torch.bfloat16, 50)])
+def test_default_tune_runs_the_default_kernel(spk, dt, K):
+    """A tune from tune_default, or one that names a compiled shape the kernel has no use for, gives the bits of
+    the call without a tune.  (The element path adds a dot's products in another order than the warp kernel.)"""
+    g = torch.Generator(device=DEV).manual_seed(K)
+    M, N, nnz = 900, 700, 12_000
+    rows = torch.randint(M, (nnz,), generator=g, device=DEV).int()
+    cols = torch.randint(N, (nnz,), generator=g, device=DEV).int()
+    S = spk.CSR.from_coo(rows, cols, (M, N), torch.rand(nnz, generator=g, device=DEV))
+    A, B = (torch.randn(n, K, generator=g, device=DEV).to(dt) for n in (M, N))
+    code = 0 if dt == torch.float32 else 1
+    e, C, X = spk.sddmm(S, A, B), spk.spmm(S, B), spk.spmm_t(S, A)
+    assert torch.equal(e, spk.sddmm(S, A, B, tune=S.tune_default(0, code, K)))
+    assert torch.equal(C, spk.spmm(S, B, tune=S.tune_default(1, code, K)))
+    assert torch.equal(X, spk.spmm_t(S, A, tune=S.tune_default(2, code, K)))
+    if K % 4:
+        assert torch.equal(e, spk.sddmm(S, A, B, tune={"variant": 2, "group_lanes": 16, "vecs_per_lane": 1, "unroll": 4}))
