@@ -71,9 +71,10 @@ typedef struct spk_tune {
     int32_t variant;        /* 0 default, 1 row-split (one lane group per row),
                                2 balanced chunks (merge-path schedule, needs spk_schedule_build),
                                  one warp per chunk, gathered rows staged in shared memory.  The
-                                 shape fields apply to SDDMM on rows of whole 16-byte vectors and
-                                 where rows are staged in registers; SpMM and rows that 16 bytes
-                                 do not divide have one layout per row width,
+                                 shape fields apply to SDDMM on rows of whole 16-byte vectors;
+                                 SpMM and rows that 16 bytes do not divide have one layout per
+                                 row width.  Rows wider than those kernels pay for are held in
+                                 registers, as in 3,
                                3 balanced chunks, gathered rows held in registers */
     int32_t group_lanes;    /* lanes that share one row of the dense factor: 4, 8, 16, 32 */
     int32_t vecs_per_lane;  /* 16-byte vectors each lane holds per K block: 1, 2, 4 */

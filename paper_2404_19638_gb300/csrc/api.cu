@@ -487,10 +487,10 @@ extern "C" spk_status spk_sddmm(spk_csr S, const float* vals, const float* vals2
     a.bnd = L.chunks ? S->bnd : nullptr;
     a.nchunks = S->nchunks;
     // rows that 16 bytes do not divide, in variant 2: the same warp kernel with
-    // smaller copies, where the rows allow 4 bytes; it has one shape per row
-    // width, so a shape that the tune names changes nothing
-    const int cb = vec || !L.ring || (int64_t)K * dt_bytes(dtb) > 512
-                       ? 0 : min(part_bytes(dta, A, lda, K), part_bytes(dtb, B, ldb, K));
+    // smaller copies, where the rows allow 4 bytes and it is the faster path; it
+    // has one shape per row width, so a shape that the tune names changes nothing
+    int cb = vec || !L.ring || (int64_t)K * dt_bytes(dtb) > 512 ? 0 : min(part_bytes(dta, A, lda, K), part_bytes(dtb, B, ldb, K));
+    if (cb && !part_sddmm_pays(dtb, cb, K, S->nnz, S->npieces > 0)) cb = 0;
     cudaError_t e = cb ? launch_sddmm_part(dta, dtb, cb, a, (cudaStream_t)stream)
                        : launch_sddmm(dta, dtb, L, a, (cudaStream_t)stream);
     if (e != cudaSuccess) return cuda_fail(e, "spk_sddmm launch");
@@ -619,7 +619,8 @@ static spk_status spmm_common(const char* name, const spk_csr_s* S, const float*
     a.meta = S->meta; a.head_s0 = S->head_s0; a.slot_np = S->slot_np; a.cnt = S->cnt;
     a.carry = reinterpret_cast<float*>(ws);
     a.nchunks = S->nchunks;
-    const int cb = vec || !L.ring ? 0 : part_bytes(dtb, B, ldb, K);
+    int cb = vec || !L.ring ? 0 : part_bytes(dtb, B, ldb, K);
+    if (cb && !part_spmm_pays(dtb, cb, K, S->nnz, S->npieces > 0)) cb = 0;
     cudaError_t e = cb ? launch_spmm_part(dtb, cb, a, stream) : launch_spmm(dtb, L, a, stream);
     if (e != cudaSuccess) return cuda_fail(e, name);
     return SPK_OK;

@@ -47,3 +47,43 @@ def test_default_tune_runs_the_default_kernel(spk, dt, K):
     assert torch.equal(X, spk.spmm_t(S, A, tune=S.tune_default(2, code, K)))
     if K % 4:
         assert torch.equal(e, spk.sddmm(S, A, B, tune={"variant": 2, "group_lanes": 16, "vecs_per_lane": 1, "unroll": 4}))
+
+
+def _skewed(spk, M, nnz, seed=0):
+    """Few rows and columns with many entries (u^3 draws), split rows among them."""
+    g = torch.Generator(device=DEV).manual_seed(seed)
+    rows, cols = ((torch.rand(nnz, generator=g, device=DEV) ** 3 * M).int().clamp_(max=M - 1) for _ in range(2))
+    return spk.CSR.from_coo(rows, cols, (M, M), torch.rand(nnz, generator=g, device=DEV))
+
+
+def _time(fn, n=8):
+    fn()
+    best = float("inf")
+    for _ in range(5):
+        e0, e1 = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+        e0.record()
+        for _ in range(n):
+            fn()
+        e1.record()
+        e1.synchronize()
+        best = min(best, e0.elapsed_time(e1))
+    return best
+
+
+@pytest.mark.parametrize("dt,K", [(torch.float32, 66), (torch.float32, 99), (torch.float32, 257), (torch.bfloat16, 130)])
+def test_wide_ragged_rows_are_no_slower_than_the_element_path(spk, dt, K):
+    """Rows of many 4- or 8-byte parts on a large skewed pattern (variant 3 is the element path): the small copies
+    took 1.8 to 3.3 times its time there."""
+    S = _skewed(spk, 1 << 17, 3_000_000)
+    B = torch.randn(S.N, K, device=DEV).to(dt)
+    assert _time(lambda: spk.spmm(S, B)) <= 1.25 * _time(lambda: spk.spmm(S, B, tune={"variant": 3}))
+
+
+@pytest.mark.parametrize("nnz,same", [(20_000, False), (1_000_000, True)])
+def test_wide_odd_sddmm_changes_path_with_the_size(spk, nnz, same):
+    """FP32 rows of 65 elements: small copies up to 2^19 entries, the element path (another order of adding) above."""
+    S = _skewed(spk, 1 << 14, nnz)
+    A, B = (torch.randn(S.M, 65, device=DEV) for _ in range(2))
+    e, r = spk.sddmm(S, A, B), spk.sddmm(S, A, B, tune={"variant": 3})
+    assert torch.equal(e, r) == same
+    torch.testing.assert_close(e, r, rtol=1e-4, atol=1e-4)
