@@ -1185,11 +1185,25 @@ extern "C" spk_status spk_spmm_t_workspace_size(spk_tplan P, int32_t K, size_t* 
     return SPK_OK;
 }
 
-static bool spmm_t_gathers_values(const spk_tplan_s* P, spk_dtype dty, const void* Y, int64_t ldy, int32_t K,
+// Whether S^T Y gathers its values through the slot permutation where the warp
+// kernel loads an index tile, or a pass puts them in CSC slot order first.  The
+// gather saves that pass and its traffic, as long as the values stay in L2 (129
+// MB) next to the gathered rows: every value is a 32-byte sector in random
+// order.  A pass of its own has L2 to itself.  Gather / pass first, GB300:
+//   rows over 128 bytes, values and rows together under 48 MB: FP32 K = 64, 2M
+//     entries 0.88-0.93 (36 MB 0.98); from 59 MB on 1.1-1.65 (8M entries, 24 a
+//     row, 0.51 / 0.33 ms), R-MAT 4M 1.14, 16M 1.36
+//   rows of 128 bytes: 16M, 24 a row, 149 MB 1.28; 8M, 75 MB 0.96; 64 bytes: 16M,
+//     8 a row, 192 MB 1.37; 107 MB 1.05; 48-96 MB 0.88-0.99; 32 bytes: 0.83-1.0
+//   the same with split rows in S^T (R-MAT 4M-30M, a few hot rows): 0.81-0.96
+static bool spmm_t_gathers_values(const spk_tplan_s* P, int arrays, spk_dtype dty, const void* Y, int64_t ldy, int32_t K,
                                   spk_dtype dtx, const void* X, int64_t ldx, const spk_tune* tune)
 {
     const int variant = (tune && tune->variant) ? tune->variant : (P->St.has_sched ? 2 : 1);
-    return variant == 2 && spmm_vec(dty, Y, ldy, K, dtx, X, ldx);
+    if (variant != 2 || !spmm_vec(dty, Y, ldy, K, dtx, X, ldx)) return false;
+    const int64_t row = (int64_t)K * dt_bytes(dty);
+    const int64_t bytes = 4 * arrays * P->St.nnz + P->M * row;
+    return row > 128 ? bytes <= 48 << 20 : (P->St.npieces > 0 || row <= 32 || bytes <= 128 << 20);
 }
 
 extern "C" spk_status spk_spmm_t(spk_tplan P, const float* vals, const float* vals2, spk_dtype dty, const void* Y,
@@ -1213,10 +1227,11 @@ extern "C" spk_status spk_spmm_t(spk_tplan P, const float* vals, const float* va
                                 nullptr, dty, Y, ldy, y_scale, K, dtx, X, ldx, accumulate, w ? w + vb : nullptr,
                                 w ? ws_bytes - vb : 0, tune, (cudaStream_t)stream, true, true);
     if (st != SPK_OK) return st;
-    // The balanced 16-byte vector path gathers the values through the
+    // The balanced 16-byte vector path can gather the values through the
     // permutation where it loads an index tile; every other path reads them
     // from the workspace in CSC slot order.
-    if (!(vals || vals2) || P->St.nnz == 0 || spmm_t_gathers_values(P, dty, Y, ldy, K, dtx, X, ldx, tune))
+    const int arrays = (vals != nullptr) + (vals2 != nullptr);
+    if (arrays == 0 || P->St.nnz == 0 || spmm_t_gathers_values(P, arrays, dty, Y, ldy, K, dtx, X, ldx, tune))
         return spmm_common("spk_spmm_t", &P->St, vals, vals2, dty, Y, ldy, y_scale, K, dtx, X, ldx, accumulate,
                            w ? w + vb : nullptr, w ? ws_bytes - vb : 0, tune, (cudaStream_t)stream);
     float* out = reinterpret_cast<float*>(w);

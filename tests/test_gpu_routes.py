@@ -87,3 +87,20 @@ def test_wide_odd_sddmm_changes_path_with_the_size(spk, nnz, same):
     e, r = spk.sddmm(S, A, B), spk.sddmm(S, A, B, tune={"variant": 3})
     assert torch.equal(e, r) == same
     torch.testing.assert_close(e, r, rtol=1e-4, atol=1e-4)
+
+
+def test_spmm_t_on_large_patterns_is_no_slower_than_permuted_values(spk):
+    """8M entries of uniform columns, values and rows of Y larger than L2: against the values gathered into CSC order
+    first and an SpMM on the transposed pattern (the gather inside the SpMM took 1.5 times as long)."""
+    M, d, K = 333_000, 24, 64
+    g = torch.Generator(device=DEV).manual_seed(3)
+    rp = (torch.arange(M + 1, device=DEV) * d).int()
+    ci = torch.randint(M, (M * d,), generator=g, device=DEV).int()
+    v = torch.rand(M * d, generator=g, device=DEV)
+    S = spk.CSR(rp, ci, (M, M), v)
+    colptr, rowidx, perm = (t.clone() for t in S.transpose_plan().arrays())
+    T = spk.CSR(colptr, rowidx, (M, M))
+    Y = torch.randn(M, K, device=DEV)
+    p = perm.long()
+    assert torch.equal(spk.spmm_t(S, Y), spk.spmm(T, Y, v[p]))
+    assert _time(lambda: spk.spmm_t(S, Y)) <= 1.15 * _time(lambda: spk.spmm(T, Y, v[p]))
