@@ -132,8 +132,8 @@ def _dw_per_head(S, dY, B, dw, heads, Kh):
         ops.sddmm(S, dY[:, c0:c0 + Kh], B[:, c0:c0 + Kh], out=dw[h], use_default_vals=False)
 
 
-def _fused_backward_steps(S, v, A, B, scores, lse, dY, R, heads, scale, softmax, need_dB):
-    """dA and dB (FP32; dB None where not needed) in separate passes: dw by one
+def _fused_backward_steps(S, v, A, B, scores, lse, dY, R, heads, scale, softmax, need_dA, need_dB):
+    """dA and dB (FP32; None where not needed) in separate passes: dw by one
     multi-head SDDMM (FP32 operands; one SDDMM per head otherwise, or where no
     multi-head kernel covers K), the score gradient c, dA = one multi-head
     SpMM, dB = two multi-head SpMM^T."""
@@ -150,7 +150,7 @@ def _fused_backward_steps(S, v, A, B, scores, lse, dY, R, heads, scale, softmax,
     else:
         _dw_per_head(S, dY, B, dw, heads, Kh)
     c = ops.fused_score_grad(S, w, dw, R, heads, softmax, scale, v)
-    dA = ops.spmm_mh(S, B, c, heads)
+    dA = ops.spmm_mh(S, B, c, heads) if need_dA else None
     dB = None
     if need_dB:
         dB = ops.spmm_t_mh(S, A, c, heads)
@@ -190,16 +190,17 @@ class FusedMMFunction(torch.autograd.Function):
         S, heads, scale, softmax = ctx.S, ctx.heads, ctx.scale, ctx.softmax
         dY = dY.contiguous().float()
         v = _vals_or_none(vals)
-        need_dB = ctx.needs_input_grad[3]
+        need_dA, need_dB = ctx.needs_input_grad[2:4]
         R = ops.fused_rowdot(dY, Y, heads) if softmax else None
         try:
-            dA, cw = ops.fused_grad(S, B, dY, scores, lse, R, heads, softmax, scale, v)
+            dA, cw = ops.fused_grad(S, B, dY, scores, lse, R, heads, softmax, scale, v, want_dA=need_dA, want_cw=need_dB)
             dB = ops.spmm_t_pair(S, cw, A, dY) if need_dB else None
         except SpkError as err:                    # no one-pass kernels for this K and these heads
             if err.code != "SPK_ERR_UNSUPPORTED":
                 raise
-            dA, dB = _fused_backward_steps(S, v, A, B, scores, lse, dY, R, heads, scale, softmax, need_dB)
-        dA = None if not ctx.needs_input_grad[2] else dA if A.dtype == torch.float32 else ops.cast(dA, A.dtype)
+            dA, dB = _fused_backward_steps(S, v, A, B, scores, lse, dY, R, heads, scale, softmax, need_dA, need_dB)
+        if dA is not None and A.dtype != torch.float32:
+            dA = ops.cast(dA, A.dtype)
         if dB is not None and B.dtype != torch.float32:
             dB = ops.cast(dB, B.dtype)
         return None, None, dA, dB, None, None, None

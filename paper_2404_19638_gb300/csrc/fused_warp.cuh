@@ -439,8 +439,11 @@ __device__ __forceinline__ void fused_warp_span(const FusedArgs& a, unsigned cha
         }
         __syncwarp();
         if constexpr (GRAD) {
-            float2* const out = reinterpret_cast<float2*>(a.cw) + (int64_t)(e0 + i) * heads;
-            for (int x = lane; x < min(left, U) * heads; x += 32) __stcs(out + x, scw[x]);
+            if (a.cw) {
+                float2* const out = reinterpret_cast<float2*>(a.cw) + (int64_t)(e0 + i) * heads;
+                for (int x = lane; x < min(left, U) * heads; x += 32) __stcs(out + x, scw[x]);
+            }
+            if (!a.Y) return;                                       // dA is not wanted: no add step
         } else if (smax && !(m & 1u)) {
             const float2 cl = scl[head];
             const f32x2 c2 = pack2(__float_as_uint(cl.x), __float_as_uint(cl.x));
@@ -494,6 +497,7 @@ __device__ __forceinline__ void fused_warp_span(const FusedArgs& a, unsigned cha
         }
     };
     auto zero_rows = [&]() {                                        // rows of the chunk without nonzeros
+        if (GRAD && !a.Y) return;
         float z[E];
 #pragma unroll
         for (int q = 0; q < E; ++q) z[q] = 0.f;
@@ -538,6 +542,7 @@ __device__ __forceinline__ void fused_warp_span(const FusedArgs& a, unsigned cha
         __syncwarp();                                               // the slot and the tile are read
     }
     cp_async_wait<0>();
+    if (GRAD && !a.Y) return;
     if (!piece && meta.y >= 0) {
         piece = 1;
         slot_id = meta.y;
