@@ -329,7 +329,7 @@ spk_status spk_fused_score_grad(spk_csr S, int32_t heads, int32_t softmax, float
  * per head, w and c as above (scores, lse: the forward's; rowdot from
  * spk_fused_rowdot; lse and rowdot only with softmax), dA_i = sum_j c B_j.
  * cw receives nnz x heads pairs (c, w), 8-byte aligned, for spk_spmm_t_pair.
- * dA or cw may be NULL where it is not wanted.  dA and dY are FP32.  Workspace: spk_fusedmm_workspace_size.  Covers rows of
+ * dA may be NULL where it is not wanted.  dA and dY are FP32.  Workspace: spk_fusedmm_workspace_size.  Covers rows of
  * B of at most 512 bytes, 16-byte aligned operands and row strides, one head
  * or heads whose columns fill a power of two of lanes; SPK_ERR_UNSUPPORTED
  * otherwise (nothing is launched). */

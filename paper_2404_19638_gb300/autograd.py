@@ -193,7 +193,7 @@ class FusedMMFunction(torch.autograd.Function):
         need_dA, need_dB = ctx.needs_input_grad[2:4]
         R = ops.fused_rowdot(dY, Y, heads) if softmax else None
         try:
-            dA, cw = ops.fused_grad(S, B, dY, scores, lse, R, heads, softmax, scale, v, want_dA=need_dA, want_cw=need_dB)
+            dA, cw = ops.fused_grad(S, B, dY, scores, lse, R, heads, softmax, scale, v, want_dA=need_dA)
             dB = ops.spmm_t_pair(S, cw, A, dY) if need_dB else None
         except SpkError as err:                    # no one-pass kernels for this K and these heads
             if err.code != "SPK_ERR_UNSUPPORTED":

@@ -773,9 +773,8 @@ extern "C" spk_status spk_fused_grad(spk_csr S, const float* scores, const float
     REQUIRE(ldb >= K && lddy >= K && ldda >= K, SPK_ERR_SHAPE, "spk_fused_grad: leading dimensions must be >= K");
     REQUIRE(stride32(ldb, dtb) && stride32(lddy, SPK_F32), SPK_ERR_SHAPE,
             "spk_fused_grad: row strides must be below 4 GiB");
-    REQUIRE(S->nnz == 0 || (B && dY && scores && (!softmax || (lse && rowdot))), SPK_ERR_ARG,
+    REQUIRE(S->nnz == 0 || (B && dY && scores && cw && (!softmax || (lse && rowdot))), SPK_ERR_ARG,
             "spk_fused_grad: NULL array");
-    REQUIRE(S->nnz == 0 || dA || cw, SPK_ERR_ARG, "spk_fused_grad: dA and cw are both NULL");
     REQUIRE((K / heads) % vec_elems(dtb) == 0 && fused_warp_supported(dtb, K, heads), SPK_ERR_UNSUPPORTED,
             "spk_fused_grad: no kernel for K = %d in %d heads", K, heads);
     REQUIRE(aligned16(B) && aligned16(dY) && aligned16(dA) && (ldb * dt_bytes(dtb)) % 16 == 0 && lddy % 4 == 0 &&

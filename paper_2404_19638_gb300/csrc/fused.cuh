@@ -13,7 +13,7 @@ cudaError_t launch_fused_mh_nv(int dt, int G, int NV, const FusedArgs& a, cudaSt
 // heads of a power of two lanes.
 bool fused_warp_supported(int dt, int K, int heads);
 cudaError_t launch_fused_warp(int dt, const FusedArgs& a, cudaStream_t s);
-// Its backward: a.A = dY (FP32), a.B the gathered factor of dtype dt, a.Y = dA; a.scores, a.lse and a.rowdot are read.
+// Its backward: a.A = dY (FP32), a.B the gathered factor of dtype dt, a.Y = dA or NULL; a.scores, a.lse and a.rowdot are read.
 cudaError_t launch_fused_grad(int dt, const FusedArgs& a, cudaStream_t s);
 
 }  // namespace spk

@@ -42,6 +42,11 @@
 
 namespace spk {
 
+// The forward; the row side of the backward; the same without dA, where only
+// the gradient of B is needed (4M rows with 1M entries, FP32 K = 64: the backward
+// 391 us with the rows of dA stored, 213 without).
+enum : int { FUSED_FORWARD = 0, FUSED_GRAD = 1, FUSED_PAIRS = 2 };
+
 // Nonzeros per batch.  A batch costs a reduction, a weight step and the loop
 // around them whatever it holds, and its slots cost resident warps; the weight
 // step of one head leaves half the lanes idle at 16.  Measured (R-MAT of 8M
@@ -57,7 +62,7 @@ constexpr int fused_warp_batch(bool grad, int row_bytes, int heads)
     return !grad && heads == 1 && row_bytes <= 128 ? 32 : 16;
 }
 
-template <int DTA, int DT, int CL, bool GRAD, int UB>
+template <int DTA, int DT, int CL, int GRAD, int UB>
 struct FusedWarp {
     static constexpr int RBB = CL * 16;                                       // bytes of a row of B, at most
     static constexpr int U = UB;
@@ -146,7 +151,7 @@ __device__ __noinline__ void fused_warp_finish(const FusedArgs& a, bool smax, in
 }
 
 // FULL: a row of B is CL * 16 bytes.
-template <int DTA, int DT, int CL, bool GRAD, int UB, bool FULL>
+template <int DTA, int DT, int CL, int GRAD, int UB, bool FULL>
 __device__ __forceinline__ void fused_warp_span(const FusedArgs& a, unsigned char* wsm, const int2 b0, const int2 b1,
                                                 const int4 meta, int head_s0)
 {
@@ -439,11 +444,9 @@ __device__ __forceinline__ void fused_warp_span(const FusedArgs& a, unsigned cha
         }
         __syncwarp();
         if constexpr (GRAD) {
-            if (a.cw) {
-                float2* const out = reinterpret_cast<float2*>(a.cw) + (int64_t)(e0 + i) * heads;
-                for (int x = lane; x < min(left, U) * heads; x += 32) __stcs(out + x, scw[x]);
-            }
-            if (!a.Y) return;                                       // dA is not wanted: no add step
+            float2* const out = reinterpret_cast<float2*>(a.cw) + (int64_t)(e0 + i) * heads;
+            for (int x = lane; x < min(left, U) * heads; x += 32) __stcs(out + x, scw[x]);
+            if constexpr (GRAD == FUSED_PAIRS) return;              // no add step
         } else if (smax && !(m & 1u)) {
             const float2 cl = scl[head];
             const f32x2 c2 = pack2(__float_as_uint(cl.x), __float_as_uint(cl.x));
@@ -497,7 +500,7 @@ __device__ __forceinline__ void fused_warp_span(const FusedArgs& a, unsigned cha
         }
     };
     auto zero_rows = [&]() {                                        // rows of the chunk without nonzeros
-        if (GRAD && !a.Y) return;
+        if (GRAD == FUSED_PAIRS) return;
         float z[E];
 #pragma unroll
         for (int q = 0; q < E; ++q) z[q] = 0.f;
@@ -542,7 +545,7 @@ __device__ __forceinline__ void fused_warp_span(const FusedArgs& a, unsigned cha
         __syncwarp();                                               // the slot and the tile are read
     }
     cp_async_wait<0>();
-    if (GRAD && !a.Y) return;
+    if (GRAD == FUSED_PAIRS) return;
     if (!piece && meta.y >= 0) {
         piece = 1;
         slot_id = meta.y;
@@ -552,7 +555,7 @@ __device__ __forceinline__ void fused_warp_span(const FusedArgs& a, unsigned cha
     if (meta.y >= 0) fused_warp_finish<E>(a, !GRAD && smax, head, lead, act, col0, meta.y, b1.x);
 }
 
-template <int DTA, int DT, int CL, bool GRAD, int UB, bool FULL>
+template <int DTA, int DT, int CL, int GRAD, int UB, bool FULL>
 __global__ void __launch_bounds__(32, CL == 8 && DT != DT_F32 ? 24 : 20)
 k_fused_warp(const FusedArgs a)
 {
@@ -564,7 +567,7 @@ k_fused_warp(const FusedArgs a)
     fused_warp_span<DTA, DT, CL, GRAD, UB, FULL>(a, ring_smem, b0, b1, m, hs0);
 }
 
-template <int DTA, int DT, int CL, bool GRAD, int UB>
+template <int DTA, int DT, int CL, int GRAD, int UB>
 cudaError_t launch_fused_warp_u(const FusedArgs& a, cudaStream_t s)
 {
     using W = FusedWarp<DTA, DT, CL, GRAD, UB>;
@@ -580,14 +583,14 @@ cudaError_t launch_fused_warp_u(const FusedArgs& a, cudaStream_t s)
     return cudaLaunchKernel(fn, dim3((unsigned)a.nchunks), dim3(32), args, smem, s);
 }
 
-template <int DTA, int DT, int CL, bool GRAD>
+template <int DTA, int DT, int CL, int GRAD>
 cudaError_t launch_fused_warp_cl(const FusedArgs& a, cudaStream_t s)
 {
     constexpr int U1 = fused_warp_batch(GRAD, CL * 16, 1), U2 = fused_warp_batch(GRAD, CL * 16, 2);
     return a.heads == 1 ? launch_fused_warp_u<DTA, DT, CL, GRAD, U1>(a, s) : launch_fused_warp_u<DTA, DT, CL, GRAD, U2>(a, s);
 }
 
-template <int DTA, int DT, bool GRAD>
+template <int DTA, int DT, int GRAD>
 cudaError_t launch_fused_warp_dt(const FusedArgs& a, cudaStream_t s)
 {
     if (a.nchunks <= 0) return cudaSuccess;

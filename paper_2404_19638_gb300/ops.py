@@ -289,10 +289,10 @@ def fused_score_grad(S: CSR, w: torch.Tensor, dw: torch.Tensor, rowdot, heads: i
 
 
 def fused_grad(S: CSR, B: torch.Tensor, dY: torch.Tensor, scores: torch.Tensor, lse, rowdot, heads: int, softmax: bool,
-               scale: float, vals=None, *, want_dA: bool = True, want_cw: bool = True):
+               scale: float, vals=None, *, want_dA: bool = True):
     """Row side of the FusedMM backward in one pass over S: (dA, cw), dA = M x K
     FP32, cw = nnz x heads x 2 pairs of the gradient c w.r.t. the unscaled dot
-    <A_i, B_j> and the weight w (None for one that is not wanted).  Raises SpkError (SPK_ERR_UNSUPPORTED) where no
+    <A_i, B_j> and the weight w (dA is None where it is not wanted).  Raises SpkError (SPK_ERR_UNSUPPORTED) where no
     kernel covers the shape or its alignment."""
     dtb, ldb = _dense(B, "B", S.device)
     dtd, lddy = _dense(dY, "dY", S.device)
@@ -304,11 +304,11 @@ def fused_grad(S: CSR, B: torch.Tensor, dY: torch.Tensor, scores: torch.Tensor, 
     rowdot = _f32(rowdot, (S.M, heads), "rowdot", S.device) if softmax else None
     vals = _vals(vals, S, "vals")
     dA = torch.empty((S.M, K), dtype=torch.float32, device=S.device) if want_dA else None
-    cw = torch.empty((S.nnz, heads, 2), dtype=torch.float32, device=S.device) if want_cw else None
+    cw = torch.empty((S.nnz, heads, 2), dtype=torch.float32, device=S.device)
     ws = S.fused_workspace(K, heads)
     check(lib().spk_fused_grad(S.handle, scores.data_ptr(), _ptr(lse), _ptr(rowdot), _ptr(vals), float(scale),
                                int(bool(softmax)), dtb, B.data_ptr(), ldb, dY.data_ptr(), lddy, K, int(heads),
-                               _ptr(dA), K, _ptr(cw), _ptr(ws), 0 if ws is None else ws.numel(),
+                               _ptr(dA), K, cw.data_ptr(), _ptr(ws), 0 if ws is None else ws.numel(),
                                _stream(S.device)), "spk_fused_grad")
     return dA, cw
 

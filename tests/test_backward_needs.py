@@ -33,8 +33,7 @@ class Recorder:
             if name == "fused_grad":
                 if not self.covered:
                     raise SpkError(next(s for s, c in STATUS.items() if c == "SPK_ERR_UNSUPPORTED"), name, "")
-                return (torch.zeros(M, K) if kw.get("want_dA", True) else None,
-                        torch.zeros(nnz, heads, 2) if kw.get("want_cw", True) else None)
+                return torch.zeros(M, K) if kw.get("want_dA", True) else None, torch.zeros(nnz, heads, 2)
             if name in ("spmm_t_pair", "spmm_t_mh"):
                 return torch.zeros(N, K)
             if name == "spmm_mh":
@@ -60,8 +59,7 @@ def test_unneeded_gradients_are_not_computed(monkeypatch, covered, heads, need_A
     assert (out[2] is not None) == need_A and (out[3] is not None) == need_B
     names = [n for n, _ in rec.calls]
     if covered:
-        kw = dict(rec.calls)["fused_grad"]
-        assert kw["want_dA"] == need_A and kw["want_cw"] == need_B
+        assert dict(rec.calls)["fused_grad"]["want_dA"] == need_A
         assert names.count("spmm_t_pair") == need_B and "spmm_mh" not in names
     else:
         assert names.count("spmm_mh") == need_A and names.count("spmm_t_mh") == 2 * need_B
