@@ -83,6 +83,26 @@ def spmm(S: CSR, B, vals=None):
     return SpMMFunction.apply(S, vals, B)
 
 
+def _one_pass(S: CSR, heads: int, row_bytes: int, need_dA: bool, need_dB: bool) -> bool:
+    """Whether the one-pass backward beats the separate steps, by size.  It saves
+    launches, gathers and (several heads) most of the traffic; with one head, on
+    large patterns without split rows, each of its two kernels holds more per
+    entry in flight and in L2 than the steps do.  Time of the one-pass kernels
+    over the steps, GB300, uniform rows of 24 / bipartite of 25: dA and dB, 8M
+    entries FP32 K = 16 1.17 / 1.08, K = 64 1.32 / 1.22, BF16 K = 128 1.25 / 1.27;
+    16M 1.13-1.36; 2M 0.65-1.1; uniform rows of 8 0.9-1.0 from 128 bytes on.  dB
+    alone, 4M FP32 K = 64 1.34 / 1.38, 8M FP32 K = 32 1.19 / 1.11; dA alone, 8M
+    K = 16 1.18 / 1.13.  4 heads 0.5-0.95 everywhere; R-MAT (split rows) 0.9-1.15."""
+    if heads > 1 or S.nnz < 3 << 20 or S.schedule_info()["npieces"] > 0:
+        return True
+    big = S.nnz >= 6 << 20
+    if row_bytes <= 64:
+        return not big
+    if need_dA:
+        return not (need_dB and big and S.nnz >= 12 * S.M)
+    return row_bytes < 256 and not big
+
+
 class GNNLayerFunction(torch.autograd.Function):
     """Y = SpMM(S_e, H) with e = SDDMM(S, H, H): an attention-style graph layer.
 
@@ -106,12 +126,19 @@ class GNNLayerFunction(torch.autograd.Function):
         S = ctx.S
         dY = dY.contiguous().float()
         v = _vals_or_none(vals)
-        try:                                       # (dE, (S.dE) H) in one pass over S, the two S^T products in another
-            acc, ee = ops.fused_grad(S, H, dY, e.reshape(1, -1), None, None, 1, False, 1.0, v)
-            ops.spmm_t_pair(S, ee, H, dY, out=acc, accumulate=True)
-        except SpkError as err:
-            if err.code != "SPK_ERR_UNSUPPORTED":
-                raise
+        acc = None
+        # the steps: FP32 rows of up to 64 bytes on large uniform patterns (16M entries, 24 a row, K = 16: 1 / 1.27 of
+        # the one-pass time; 8 a row 1 / 1.01; wider and 16-bit rows gain by the one pass)
+        if not (H.dtype == torch.float32 and H.size(1) <= 16 and S.has_schedule
+                and not _one_pass(S, 1, 4 * H.size(1), True, False)):
+            try:                                   # (dE, (S.dE) H) in one pass over S, the two S^T products in another
+                acc, ee = ops.fused_grad(S, H, dY, e.reshape(1, -1), None, None, 1, False, 1.0, v)
+                ops.spmm_t_pair(S, ee, H, dY, out=acc, accumulate=True)
+            except SpkError as err:
+                if err.code != "SPK_ERR_UNSUPPORTED":
+                    raise
+                acc = None
+        if acc is None:
             dE = ops.sddmm(S, dY, H, use_default_vals=False)
             acc = ops.spmm(S, H, v, dE, use_default_vals=False)
             ops.spmm_t(S, H, v, dE, out=acc, accumulate=True, use_default_vals=False)
@@ -170,8 +197,9 @@ class FusedMMFunction(torch.autograd.Function):
     Steps: the row term; one pass over S that gathers B once for dw, the
     weights, c and dA (ops.fused_grad); one pass over S^T that adds both
     products of dB to one output (ops.spmm_t_pair), all heads at once, in
-    FP32.  Where those kernels don't cover K, the heads or the alignment, the
-    same steps one by one (_fused_backward_steps).  The sparse values are not
+    FP32.  Where those kernels don't cover K, the heads or the alignment, or are
+    the slower way (_one_pass), the same steps one by one
+    (_fused_backward_steps).  The sparse values are not
     differentiated.
     """
 
@@ -192,12 +220,16 @@ class FusedMMFunction(torch.autograd.Function):
         v = _vals_or_none(vals)
         need_dA, need_dB = ctx.needs_input_grad[2:4]
         R = ops.fused_rowdot(dY, Y, heads) if softmax else None
-        try:
-            dA, cw = ops.fused_grad(S, B, dY, scores, lse, R, heads, softmax, scale, v, want_dA=need_dA)
-            dB = ops.spmm_t_pair(S, cw, A, dY) if need_dB else None
-        except SpkError as err:                    # no one-pass kernels for this K and these heads
-            if err.code != "SPK_ERR_UNSUPPORTED":
-                raise
+        done = False
+        if _one_pass(S, heads, B.size(1) * B.element_size(), need_dA, need_dB):
+            try:
+                dA, cw = ops.fused_grad(S, B, dY, scores, lse, R, heads, softmax, scale, v, want_dA=need_dA)
+                dB = ops.spmm_t_pair(S, cw, A, dY) if need_dB else None
+                done = True
+            except SpkError as err:                # no one-pass kernels for this K and these heads
+                if err.code != "SPK_ERR_UNSUPPORTED":
+                    raise
+        if not done:
             dA, dB = _fused_backward_steps(S, v, A, B, scores, lse, dY, R, heads, scale, softmax, need_dA, need_dB)
         if dA is not None and A.dtype != torch.float32:
             dA = ops.cast(dA, A.dtype)

@@ -45,6 +45,10 @@ class Recorder:
         return call
 
 
+def _pattern(M, nnz, npieces=0):
+    return types.SimpleNamespace(M=M, nnz=nnz, has_schedule=True, schedule_info=lambda: {"npieces": npieces})
+
+
 @pytest.mark.parametrize("need_A,need_B", NEEDS)
 @pytest.mark.parametrize("covered,heads", [(True, 2), (False, 2), (False, 1)])
 def test_unneeded_gradients_are_not_computed(monkeypatch, covered, heads, need_A, need_B):
@@ -53,7 +57,7 @@ def test_unneeded_gradients_are_not_computed(monkeypatch, covered, heads, need_A
     monkeypatch.setattr(ag, "ops", rec)
     A, B, Y = torch.zeros(M, K), torch.zeros(N, K), torch.zeros(M, K)
     ctx = types.SimpleNamespace(saved_tensors=(torch.empty(0), A, B, Y, torch.zeros(heads, nnz), torch.zeros(M, heads)),
-                                S=types.SimpleNamespace(nnz=nnz), heads=heads, scale=1.0, softmax=True,
+                                S=_pattern(M, nnz), heads=heads, scale=1.0, softmax=True,
                                 needs_input_grad=(False, False, need_A, need_B, False, False, False))
     out = ag.FusedMMFunction.backward(ctx, torch.ones(M, K))
     assert (out[2] is not None) == need_A and (out[3] is not None) == need_B
@@ -63,6 +67,23 @@ def test_unneeded_gradients_are_not_computed(monkeypatch, covered, heads, need_A
         assert names.count("spmm_t_pair") == need_B and "spmm_mh" not in names
     else:
         assert names.count("spmm_mh") == need_A and names.count("spmm_t_mh") == 2 * need_B
+
+
+@pytest.mark.parametrize("M,nnz,pieces,heads,K,needs,one", [
+    (1 << 19, 12 << 20, 0, 1, 64, (True, True), False), (1 << 19, 12 << 20, 9, 1, 64, (True, True), True),
+    (1 << 19, 12 << 20, 0, 2, 64, (True, True), True), (1 << 22, 12 << 20, 0, 1, 64, (True, True), True),
+    (1 << 22, 12 << 20, 0, 1, 16, (True, True), False), (1 << 18, 4 << 20, 0, 1, 64, (True, True), True),
+    (1 << 18, 4 << 20, 0, 1, 64, (False, True), False), (1 << 18, 4 << 20, 0, 1, 32, (False, True), True),
+    (1 << 19, 12 << 20, 0, 1, 64, (True, False), True), (1 << 19, 12 << 20, 0, 1, 16, (True, False), False)])
+def test_one_pass_or_steps_by_size(monkeypatch, M, nnz, pieces, heads, K, needs, one):
+    rec = Recorder(True, 2, 2, K, 1, heads)
+    monkeypatch.setattr(ag, "ops", rec)
+    X = torch.zeros(2, K)
+    ctx = types.SimpleNamespace(saved_tensors=(torch.empty(0), X, X, X, torch.zeros(heads, 1), torch.zeros(2, heads)),
+                                S=_pattern(M, nnz, pieces), heads=heads, scale=1.0, softmax=True,
+                                needs_input_grad=(False, False, *needs, False, False, False))
+    ag.FusedMMFunction.backward(ctx, X)
+    assert ("fused_grad" in [n for n, _ in rec.calls]) == one
 
 
 @pytest.fixture(scope="module")
