@@ -1,8 +1,9 @@
 """Autotuner for the kernel schedule of one sparse pattern.
 
-The fastest lane-group shape (lanes per dense row, 16-byte vectors per lane,
-nonzeros in flight), CTA size and balanced-schedule chunk size depend on the
-degree distribution of S, on K and on the dtype.  Following the paper's
+The fastest kernel (the warp kernels or the register path), its lane-group
+shape where it has one (lanes per dense row, 16-byte vectors per lane, nonzeros
+in flight), CTA size and balanced-schedule chunk size depend on the degree
+distribution of S, on K and on the dtype.  Following the paper's
 "set up once, run many times" structure (Sec. 5.1: the pattern is fixed while
 values change), the tuner times a small set of candidates once per
 (pattern, op, dtype, K) with CUDA events on the current stream, keeps the
@@ -26,6 +27,10 @@ import torch
 from . import ops
 from .binding import SpkError
 from .sparse import CSR
+
+# Part of every cache key, raised when the kernels behind the tunes change: an
+# entry chosen among other kernels is timed again.
+CACHE_VERSION = 2
 
 _VEC = {torch.float32: 4, torch.bfloat16: 8, torch.float16: 8, torch.float8_e4m3fn: 16, torch.uint8: 16}
 
@@ -52,6 +57,18 @@ def candidate_shapes(K: int, dtype) -> list[tuple[int, int, int]]:
         if cover >= nvec and cover <= max(4, 2 * nvec):
             out.append((G, NV, U))
     return out or [(32, 4, 4)]
+
+
+def candidate_tunes(op: str, K: int, dtype, threads=(128, 256)) -> list[dict]:
+    """Balanced candidates, each a kernel of its own, the one a call without a
+    tune runs first: the warp kernels (variant 2; SDDMM on rows of whole 16-byte
+    vectors has a shape to choose there, the others have one layout per row
+    width), then the register path in every shape and CTA size."""
+    shapes = [{"group_lanes": G, "vecs_per_lane": NV, "unroll": U} for G, NV, U in candidate_shapes(K, dtype)]
+    warp = [{"variant": 2}]
+    if op == "sddmm" and K % _VEC.get(dtype, 4) == 0:
+        warp += [{"variant": 2, **s} for s in shapes]
+    return warp + [{"variant": 3, **s, "cta_threads": thr} for s in shapes for thr in threads]
 
 
 class Autotuner:
@@ -85,7 +102,7 @@ class Autotuner:
     @staticmethod
     def key(S: CSR, op: str, dtype, K: int) -> str:
         sig = pattern_signature(S.rowptr.cpu().numpy(), S.M, S.N)
-        return f"{sig}|{op}|{str(dtype).replace('torch.', '')}|{K}"
+        return f"{CACHE_VERSION}|{sig}|{op}|{str(dtype).replace('torch.', '')}|{K}"
 
     def lookup(self, S: CSR, op: str, dtype, K: int) -> dict | None:
         return self._cache.get(self.key(S, op, dtype, K))
@@ -139,18 +156,13 @@ class Autotuner:
         best = None
         for W in self.chunk_works:
             self._attach(S, op, W)
-            for (G, NV, U) in candidate_shapes(K, dtype):
-                # shared-memory ring (2 or 4 slots), then the register path at each CTA size
-                cands = [{"variant": 2, "stages": st} for st in (2, 4)]
-                cands += [{"variant": 3, "cta_threads": thr} for thr in self.threads]
-                for c in cands:
-                    t = {"group_lanes": G, "vecs_per_lane": NV, "unroll": U, **c}
-                    try:
-                        ms = self._time(lambda: run(t))
-                    except SpkError:
-                        continue
-                    if best is None or ms < best["ms"]:
-                        best = {"tune": t, "chunk_work": W, "ms": ms}
+            for t in candidate_tunes(op, K, dtype, self.threads):
+                try:
+                    ms = self._time(lambda: run(t))
+                except SpkError:
+                    continue
+                if best is None or ms < best["ms"]:
+                    best = {"tune": t, "chunk_work": W, "ms": ms}
         # the row-split variant, for patterns without long rows
         for (G, NV, U) in candidate_shapes(K, dtype)[:2]:
             t = {"variant": 1, "group_lanes": G, "vecs_per_lane": NV, "unroll": U, "cta_threads": self.threads[0]}
@@ -169,4 +181,4 @@ class Autotuner:
         return best
 
 
-__all__ = ["Autotuner", "pattern_signature", "candidate_shapes"]
+__all__ = ["Autotuner", "pattern_signature", "candidate_shapes", "candidate_tunes"]
