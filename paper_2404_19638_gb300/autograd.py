@@ -83,6 +83,12 @@ def spmm(S: CSR, B, vals=None):
     return SpMMFunction.apply(S, vals, B)
 
 
+def _one_pass_rows(row_bytes: int) -> bool:
+    """Rows of B that the one-pass kernels may cover.  Others are not tried: the call that refuses them comes after
+    its outputs are allocated, 20-40 us of host time."""
+    return row_bytes <= 512 and row_bytes % 16 == 0
+
+
 def _one_pass(S: CSR, heads: int, row_bytes: int, need_dA: bool, need_dB: bool) -> bool:
     """Whether the one-pass backward beats the separate steps, by size.  It saves
     launches, gathers and (several heads) most of the traffic; with one head, on
@@ -93,6 +99,8 @@ def _one_pass(S: CSR, heads: int, row_bytes: int, need_dA: bool, need_dB: bool) 
     16M 1.13-1.36; 2M 0.65-1.1; uniform rows of 8 0.9-1.0 from 128 bytes on.  dB
     alone, 4M FP32 K = 64 1.34 / 1.38, 8M FP32 K = 32 1.19 / 1.11; dA alone, 8M
     K = 16 1.18 / 1.13.  4 heads 0.5-0.95 everywhere; R-MAT (split rows) 0.9-1.15."""
+    if not _one_pass_rows(row_bytes):
+        return False
     if heads > 1 or S.nnz < 3 << 20 or S.schedule_info()["npieces"] > 0:
         return True
     big = S.nnz >= 6 << 20
@@ -129,8 +137,9 @@ class GNNLayerFunction(torch.autograd.Function):
         acc = None
         # the steps: FP32 rows of up to 64 bytes on large uniform patterns (16M entries, 24 a row, K = 16: 1 / 1.27 of
         # the one-pass time; 8 a row 1 / 1.01; wider and 16-bit rows gain by the one pass)
-        if not (H.dtype == torch.float32 and H.size(1) <= 16 and S.has_schedule
-                and not _one_pass(S, 1, 4 * H.size(1), True, False)):
+        row_bytes = H.size(1) * H.element_size()
+        if S.has_schedule and _one_pass_rows(row_bytes) and (H.dtype != torch.float32 or H.size(1) > 16
+                                                             or _one_pass(S, 1, row_bytes, True, False)):
             try:                                   # (dE, (S.dE) H) in one pass over S, the two S^T products in another
                 acc, ee = ops.fused_grad(S, H, dY, e.reshape(1, -1), None, None, 1, False, 1.0, v)
                 ops.spmm_t_pair(S, ee, H, dY, out=acc, accumulate=True)

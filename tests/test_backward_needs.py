@@ -86,6 +86,24 @@ def test_one_pass_or_steps_by_size(monkeypatch, M, nnz, pieces, heads, K, needs,
     assert ("fused_grad" in [n for n, _ in rec.calls]) == one
 
 
+@pytest.mark.parametrize("K,tried", [(128, True), (132, False), (50, False)])
+def test_rows_that_no_one_pass_kernel_covers_are_not_tried(monkeypatch, K, tried):
+    rec = Recorder(True, 2, 2, K, 1, 1)
+    monkeypatch.setattr(ag, "ops", rec)
+    X = torch.zeros(2, K)
+    need = (False, False, True, True, False, False, False)
+    ctx = types.SimpleNamespace(saved_tensors=(torch.empty(0), X, X, X, torch.zeros(1, 1), torch.zeros(2, 1)),
+                                S=_pattern(2, 1), heads=1, scale=1.0, softmax=True, needs_input_grad=need)
+    ag.FusedMMFunction.backward(ctx, X)
+    assert ("fused_grad" in [n for n, _ in rec.calls]) == tried
+    rec.calls.clear()
+    monkeypatch.setattr(rec, "sddmm", lambda *a, **k: None, raising=False)
+    monkeypatch.setattr(rec, "spmm", lambda *a, **k: X, raising=False)
+    ctx = types.SimpleNamespace(saved_tensors=(torch.empty(0), X, torch.zeros(1)), S=_pattern(2, 1))
+    ag.GNNLayerFunction.backward(ctx, X)
+    assert ("fused_grad" in [n for n, _ in rec.calls]) == tried
+
+
 @pytest.fixture(scope="module")
 def spk():
     if not torch.cuda.is_available():
