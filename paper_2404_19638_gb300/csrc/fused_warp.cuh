@@ -555,8 +555,27 @@ __device__ __forceinline__ void fused_warp_span(const FusedArgs& a, unsigned cha
     if (meta.y >= 0) fused_warp_finish<E>(a, !GRAD && smax, head, lead, act, col0, meta.y, b1.x);
 }
 
+// Resident warps an SM that the registers are cut for.  More warps hide the
+// latency of the gathers and of the serial steps of a batch, where shared memory
+// has room for them (about 30 on rows of 64 bytes, 27 on 128 with several heads);
+// with 18 in shared memory (128 bytes and one head, 256 bytes) the limit only
+// changes the code.  Time over that at 20 warps (R-MAT of 4M and 8M entries, regular rows of 8 and
+// 24, no spills): forward, rows of up to 64 bytes at 24 warps 0.82-0.95, at 32
+// 0.80-0.92 (one head or two, FP32 and BF16); 128 bytes, FP32 at 24 0.97 one
+// head, 0.82-0.88 two, at 28 1.0 / 0.82-0.9; BF16 at 24 0.98 one head, 0.82-0.94
+// four, at 28 another 0.95; 256 bytes, BF16 at 24 0.92-0.97, FP32 0.99-1.01.
+// Backward: up to 64 bytes at 24 0.98-1.12, at 32 0.92-1.12; BF16 rows of 128
+// bytes at 28 1.03-1.06 of 24.
+constexpr int fused_warp_ctas(bool grad, int dt, int cl)
+{
+    if (grad) return cl == 8 && dt != DT_F32 ? 24 : 20;
+    if (cl <= 4) return 32;
+    if (cl == 8) return dt != DT_F32 ? 28 : 24;
+    return cl == 16 && dt != DT_F32 ? 24 : 20;
+}
+
 template <int DTA, int DT, int CL, int GRAD, int UB, bool FULL>
-__global__ void __launch_bounds__(32, CL == 8 && DT != DT_F32 ? 24 : 20)
+__global__ void __launch_bounds__(32, fused_warp_ctas(GRAD != FUSED_FORWARD, DT, CL))
 k_fused_warp(const FusedArgs a)
 {
     extern __shared__ __align__(16) unsigned char ring_smem[];
