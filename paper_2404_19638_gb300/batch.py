@@ -116,7 +116,7 @@ class Batch:
         the chunk size of each group of patterns of similar size (nonzeros
         within a factor of 4), largest patterns first; the shape (group
         lanes, vectors per lane, nonzeros per batch; spk_batch_shapes) of
-        each class of items of one op, K and dtype; the kernel's register
+        each class of SDDMM items of one K and dtype; the kernel's register
         budget (80 or 96).  Returns {"chunk_work": W, "ms": {W: ms}} plus,
         with per_item, "chunk_work_by_nnz", "shapes", "registers", "ms_final"
         and "trials" (whole launches timed after the first stage, each
@@ -171,7 +171,7 @@ class Batch:
             now = ((t0.group_lanes, t0.vecs_per_lane, t0.unroll) if t0 is not None and t0.group_lanes
                    else (4 if nvec <= 4 else (8 if nvec <= 8 else 16), 1, 4))
             chosen = None
-            for G, NV, U in batch_shapes(op):
+            for G, NV, U in batch_shapes(op) if op == OP_SDDMM else ():      # an SpMM item's routine follows K alone
                 if G * NV < nvec or (G, NV, U) == now:
                     continue
                 for k in ks:

@@ -86,9 +86,13 @@ __device__ __noinline__ void batch_spmm_unit(const SpmmArgs& a, int64_t c, unsig
     else spmm_warp_span<DT, CL, SPMM_STORE, false>(a, wsm, 0, 1, b0, b1, m, hs0);
 }
 
-// MINB: CTAs per SM the register budget is cut for (6: 80 registers; 5: 96
-// registers, for batches with 8-nonzero SpMM batches or BF16 operands, whose
-// routines would spill at 80).
+// MINB: CTAs per SM the register budget is cut for (6: 80 registers, the
+// default; 5: 96 registers, on request).  No routine spills at 80, and the sixth
+// CTA pays: SDDMM + SpMM of 64 matrices with 24 a row, 30M nonzeros in all, 80 /
+// 96 registers, FP32 K = 16 / 32 / 64 739 / 809, 897 / 972, 1221 / 1300 us, BF16
+// K = 16 / 32 / 64 / 128 824 / 952, 758 / 854, 1018 / 1094, 1565 / 1569 us.  Small
+// batches (1M nonzeros, about 50 us) are equal; one op alone runs up to 10 %
+// faster with 96 there.
 template <int MINB>
 __global__ void __launch_bounds__(kBatchThreads, MINB) k_batch(const BatchDesc* __restrict__ descs, int32_t count,
                                                   const int64_t* __restrict__ unit_begin, int64_t total_units,
@@ -151,8 +155,7 @@ struct spk_batch_s {
     int64_t total_units;
     int32_t grid;
     int32_t ring_bytes;              // per warp: the largest ring among the items' shapes
-    bool wide;                       // the 96-register kernel build (see plan_batch)
-    bool wide_default;               // the build plan_batch chose
+    bool wide;                       // the 96-register kernel build
     const BatchDesc* d_descs;
     const int64_t* d_unit_begin;
     unsigned long long* d_counter;
@@ -174,7 +177,6 @@ struct BatchPlan {
     size_t off_descs, off_units, off_counter, off_done, off_carry, total;
     std::vector<size_t> carry_off;   // per item (SpMM), relative to off_carry
     int ring_bytes = 0;              // per warp
-    bool wide = false;               // some item batches 8 nonzeros or has BF16 operands
 };
 
 static spk_status plan_batch(const spk_batch_item* items, int32_t count, BatchPlan& P)
@@ -240,7 +242,6 @@ static spk_status plan_batch(const spk_batch_item* items, int32_t count, BatchPl
         const int cl = nvec <= 4 ? 4 : (nvec <= 8 ? 8 : 16);         // SpMM: 16-byte vectors per gathered row
         const int rb = batch_ring_bytes(it.op, list[sidx], cl);
         if (rb > P.ring_bytes) P.ring_bytes = rb;
-        if (list[sidx].U > 4 || it.dt == SPK_BF16) P.wide = true;
         BatchDesc& d = P.descs[m];
         d.op = it.op;
         d.cls = it.op == 0 ? (it.dt == SPK_BF16 ? 8 : 0) + sidx : (it.dt == SPK_BF16 ? 32 : 0) + cl;
@@ -331,7 +332,7 @@ extern "C" spk_status spk_batch_create(const spk_batch_item* items, int32_t coun
     if (e == cudaSuccess) e = cudaStreamSynchronize(cs);
     if (e != cudaSuccess) return bfail(SPK_ERR_CUDA, std::string("spk_batch_create: ") + cudaGetErrorString(e));
     int grid = 0;
-    e = batch_grid(P.wide, P.ring_bytes, &grid);
+    e = batch_grid(false, P.ring_bytes, &grid);
     if (e != cudaSuccess) return bfail(SPK_ERR_CUDA, std::string("spk_batch_create: ") + cudaGetErrorString(e));
     spk_batch_s* B = new (std::nothrow) spk_batch_s();
     if (!B) return bfail(SPK_ERR_ARG, "spk_batch_create: out of host memory");
@@ -339,8 +340,7 @@ extern "C" spk_status spk_batch_create(const spk_batch_item* items, int32_t coun
     B->total_units = P.unit_begin[count];
     B->grid = grid;
     B->ring_bytes = P.ring_bytes;
-    B->wide = P.wide;
-    B->wide_default = P.wide;
+    B->wide = false;
     B->d_descs = reinterpret_cast<const BatchDesc*>(st + P.off_descs);
     B->d_unit_begin = reinterpret_cast<const int64_t*>(st + P.off_units);
     B->d_counter = reinterpret_cast<unsigned long long*>(st + P.off_counter);
@@ -385,7 +385,7 @@ extern "C" spk_status spk_batch_set_registers(spk_batch B, int32_t regs)
     if (!B) return bfail(SPK_ERR_ARG, "spk_batch_set_registers: handle is NULL");
     if (regs != 0 && regs != 80 && regs != 96)
         return bfail(SPK_ERR_ARG, "spk_batch_set_registers: regs must be 0, 80 or 96");
-    const bool wide = regs == 0 ? B->wide_default : regs == 96;
+    const bool wide = regs == 96;
     int grid = 0;
     cudaError_t e = batch_grid(wide, B->ring_bytes, &grid);
     if (e != cudaSuccess) return bfail(SPK_ERR_CUDA, std::string("spk_batch_set_registers: ") + cudaGetErrorString(e));

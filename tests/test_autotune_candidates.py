@@ -1,11 +1,12 @@
-"""What the tuner times: the call without a tune among the candidates, and no
-kernel twice (host logic, with the launches replaced by a recorder)."""
+"""What the tuners time: the call without a tune among the candidates, and no
+kernel twice (host logic, with the launches replaced by recorders)."""
 import types
 
 import pytest
 import torch
 
 import paper_2404_19638_gb300.autotune as at
+from paper_2404_19638_gb300 import Batch, Item, OP_SDDMM, OP_SPMM
 
 
 def _pattern(M, N, nnz):
@@ -47,3 +48,20 @@ def test_cache_entries_of_other_kernels_are_not_found(tmp_path):
     sig = at.pattern_signature(S.rowptr.numpy(), S.M, S.N)
     tuner._cache[f"{sig}|sddmm|float32|50"] = {"tune": {"variant": 2, "group_lanes": 16}, "chunk_work": 512, "ms": 1.0}
     assert tuner.lookup(S, "sddmm", torch.float32, 50) is None
+
+
+def test_batch_tunes_shapes_of_sddmm_items_only(monkeypatch):
+    """A batched SpMM item has one routine per row width: nothing to choose."""
+    S = _pattern(40, 30, 200)
+    A, B = torch.empty(40, 32), torch.empty(30, 32)
+    b = Batch.__new__(Batch)
+    b.items = [Item(OP_SDDMM, S, B, torch.empty(200), A=A), Item(OP_SPMM, S, B, torch.empty(40, 32))]
+    b._tunes, b._h = [None, None], None
+    tuned = []
+    for name, f in (("_create", lambda self: None), ("_destroy", lambda self: None), ("__del__", lambda self: None),
+                    ("_time", lambda self, reps: 1.0), ("set_registers", lambda self, r: None),
+                    ("set_item_tune", lambda self, k, t: tuned.append((k, t)))):
+        monkeypatch.setattr(Batch, name, f)
+    b.autotune((64, 128), per_item=True)
+    assert any(k == 0 and t is not None for k, t in tuned)
+    assert all(t is None for k, t in tuned if k == 1)

@@ -104,3 +104,20 @@ def test_spmm_t_on_large_patterns_is_no_slower_than_permuted_values(spk):
     p = perm.long()
     assert torch.equal(spk.spmm_t(S, Y), spk.spmm(T, Y, v[p]))
     assert _time(lambda: spk.spmm_t(S, Y)) <= 1.15 * _time(lambda: spk.spmm(T, Y, v[p]))
+
+
+@pytest.mark.parametrize("dt", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("tune", [None, {"group_lanes": 8, "vecs_per_lane": 1, "unroll": 8}])
+def test_batch_runs_six_ctas_an_sm(spk, dt, tune):
+    """Neither BF16 operands nor a shape named for SpMM (one routine per row width) cost resident warps."""
+    S = _skewed(spk, 3000, 40_000)
+    B = torch.randn(S.N, 32, device=DEV).to(dt)
+    out = torch.empty(S.M, 32, device=DEV)
+    b = spk.Batch([spk.Item(spk.OP_SPMM, S, B, out, tune=tune)])
+    b.run()
+    assert torch.equal(out, spk.spmm(S, B))
+    default = b.info()
+    b.set_registers(80)
+    assert b.info() == default
+    b.set_registers(96)
+    assert b.info()["ctas"] < default["ctas"]
