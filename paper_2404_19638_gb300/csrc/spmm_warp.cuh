@@ -404,7 +404,7 @@ __device__ __forceinline__ void spmm_warp_span(const SpmmArgs& a, unsigned char*
                 zm &= zm - 1;
                 if (!act) continue;
                 if constexpr (CB < 16) write_some_at<E>(a, p, z, ne, celt);
-                else if constexpr (MODE == SPMM_ANY) write_vec_at<E>(a, p, z);
+                else if constexpr (MODE == SPMM_ANY) store_elems<DT_BF16, E>(p, 0, z);      // BF16 and F16 zeros are the same bits
                 else store_elems<DT_F32, E>(p, 0, z);
             }
         }
