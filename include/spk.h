@@ -74,7 +74,8 @@ typedef struct spk_tune {
                                  shape fields apply to SDDMM on rows of whole 16-byte vectors;
                                  SpMM and rows that 16 bytes do not divide have one layout per
                                  row width.  Rows wider than those kernels pay for are held in
-                                 registers, as in 3,
+                                 registers, as in 3, and SpMM of FP32 rows of at most 64 bytes on
+                                 large patterns of rows of nearly one length is split by rows, as in 1,
                                3 balanced chunks, gathered rows held in registers */
     int32_t group_lanes;    /* lanes that share one row of the dense factor: 4, 8, 16, 32 */
     int32_t vecs_per_lane;  /* 16-byte vectors each lane holds per K block: 1, 2, 4 */

@@ -175,13 +175,15 @@ static spk_status attach_schedule(spk_csr_s* S, int32_t W, void* storage, size_t
             "schedule storage must be 256-byte aligned");
     char* st = reinterpret_cast<char*>(storage);
     int64_t np = 0;
+    bool regular = false;
     S->has_sched = false;
-    cudaError_t e = build_schedule(S->rowptr, S->M, S->nnz, W, st, L, &np, s);
+    cudaError_t e = build_schedule(S->rowptr, S->M, S->nnz, W, st, L, &np, &regular, s);
     if (e != cudaSuccess) return cuda_fail(e, "schedule build");
     S->has_sched = true;
     S->W = W;
     S->nchunks = L.nchunks;
     S->npieces = np;
+    S->regular = regular;
     S->rowidx = reinterpret_cast<const int32_t*>(st + L.rowidx);
     S->bnd = reinterpret_cast<const int2*>(st + L.bnd);
     S->meta = reinterpret_cast<const int4*>(st + L.meta);
@@ -552,6 +554,19 @@ extern "C" spk_status spk_spmm_workspace_size(spk_csr S, int32_t K, size_t* byte
 
 // 16-byte vectors throughout: whole vectors a row, aligned rows of B and C.
 static bool spmm_vec(spk_dtype dtb, const void* B, int64_t ldb, int32_t K, spk_dtype dtc, const void* C, int64_t ldc)
+// Whether FP32 rows of at most 64 bytes run row-split instead of the balanced
+// warp kernel, which has work for half its lanes or fewer there.  Where all rows
+// are nearly of one length the split balances by itself and the lane groups of a
+// warp change rows together; on other patterns the warp kernel is the faster or
+// the safer one.  Row-split / warp kernel / the lane-group ring before both, us:
+//   14M entries, 24 a row, K = 4 / 8 / 16 77 / 154 / 121, 77 / 150 / 122, 81 / 158 / 107;
+//   8M, 24 a row, K = 16 47 / 94 / 88; 14M, 30 or 31 a row 126 / 156 / 119; 12M, 20
+//   or 21 113 / 143 / 125; 8.5M, 8 or 9 136 / 115 / 136; 8M, 4 a row 142 / 138 / 130.
+static bool spmm_row_split_pays(const spk_csr_s* S, int dt, int K)
+{
+    return dt == SPK_F32 && K <= 16 && S->regular && !S->vperm && S->nnz >= 6 << 20 && S->nnz >= 12 * S->M;
+}
+
 {
     return (K % vec_elems(dtb)) == 0 && aligned16(B) && aligned16(C) && (ldb * dt_bytes(dtb)) % 16 == 0 &&
            (ldc * dt_bytes(dtc)) % 16 == 0;
@@ -614,6 +629,11 @@ static spk_status spmm_common(const char* name, const spk_csr_s* S, const float*
     a.heads = heads;
     a.hstride = hstride;
     a.B = B; a.ldb = ldb; a.b_scale = b_scale;
+    if (vec && L.ring && heads == 1 && spmm_row_split_pays(S, dtb, K)) {
+        a.bnd = nullptr;
+        L.chunks = L.ring = false;
+        L.shape = shape_index(4, 1, 4);
+    }
     a.C = C; a.ldc = ldc; a.dtc = dtc; a.accumulate = accumulate;
     a.bnd = L.chunks ? S->bnd : nullptr;
     a.meta = S->meta; a.head_s0 = S->head_s0; a.slot_np = S->slot_np; a.cnt = S->cnt;

@@ -411,7 +411,7 @@ SchedLayout sched_layout(int64_t M, int64_t nnz, int32_t W);
 size_t scan_temp_bytes(int64_t n);
 cudaError_t scan_exclusive_i32(const int32_t* in, int32_t* out, int64_t n, void* tmp, cudaStream_t s);
 cudaError_t build_schedule(const int32_t* rowptr, int64_t M, int64_t nnz, int32_t W, char* storage,
-                           const SchedLayout& L, int64_t* npieces_out, cudaStream_t s);
+                           const SchedLayout& L, int64_t* npieces_out, bool* regular_out, cudaStream_t s);
 cudaError_t launch_validate(const int32_t* rowptr, const int32_t* colidx, int64_t M, int64_t N, int64_t nnz,
                             int32_t* report, cudaStream_t s);
 
@@ -511,6 +511,7 @@ struct spk_csr_s {
     // balanced schedule (in caller storage)
     bool has_sched;
     int32_t W;
+    bool regular;             // rows of nearly one length, none split
     int64_t nchunks, npieces;
     const int32_t* rowidx;
     const int2* bnd;

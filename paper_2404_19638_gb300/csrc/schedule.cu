@@ -115,7 +115,7 @@ SchedLayout sched_layout(int64_t M, int64_t nnz, int32_t W)
     L.head_s0 = off;  off += align256((size_t)L.nchunks * 4);
     L.slot_np = off;  off += align256((size_t)L.nchunks * 8 + 4);
     L.cnt = off;      off += align256((size_t)L.nchunks * 8 + 4);
-    L.pieces = off;   off += align256((size_t)(L.nchunks + 1) * 4);
+    L.pieces = off;   off += align256((size_t)(L.nchunks + 2) * 4);
     L.scan_tmp = off; off += align256(scan_temp_bytes(L.nchunks + 1));
     L.total = off;
     return L;
@@ -166,11 +166,19 @@ __device__ __forceinline__ void chunk_flags(const int2* bnd, const int32_t* rowp
     r_last = ends_inside ? b1.x : b1.x - 1;
 }
 
-__global__ void k_sched_pieces(const int2* bnd, const int32_t* rowptr, int64_t M, int64_t nchunks,
+// pieces[nchunks + 1] is set where some boundary lies off the line on which it
+// would lie if all rows had one length, by more than a tenth of sqrt(nnz) entries
+// (random row lengths come several times as far), so that kernels whose lane
+// groups take rows of their own can tell patterns on which they keep in step.
+__global__ void k_sched_pieces(const int2* bnd, const int32_t* rowptr, int64_t M, int64_t nnz, int64_t nchunks,
                                int32_t* pieces)
 {
     const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (c > nchunks) return;
+    if (nnz > 0) {
+        const int r = bnd[c].x;
+        if (fabs((double)rowptr[r] - (double)r * (double)nnz / (double)M) > 0.1 * sqrt((double)nnz)) pieces[nchunks + 1] = 1;
+    }
     if (c == nchunks) { pieces[c] = 0; return; }
     int head, tail, r_last;
     chunk_flags(bnd, rowptr, M, c, head, tail, r_last);
@@ -239,9 +247,10 @@ __device__ __forceinline__ int64_t row_of_entry_warp(const int32_t* rowptr, int6
 constexpr int COO_SPAN = 256, COO_WARPS = 8;
 
 __global__ void __launch_bounds__(32 * COO_WARPS) k_coo_rows(const int32_t* __restrict__ rowptr, int64_t M, int64_t nnz,
-                                                            int32_t* __restrict__ rowidx)
+                                                            int32_t* __restrict__ rowidx, int32_t* irregular)
 {
     __shared__ int32_t mark[COO_WARPS][COO_SPAN];
+    if (blockIdx.x == 0 && threadIdx.x == 0) *irregular = 0;         // set by k_sched_pieces
     const int64_t e0 = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * COO_SPAN;
     if (e0 >= nnz) return;
     const int lane = threadIdx.x & 31;
@@ -277,7 +286,7 @@ __global__ void __launch_bounds__(32 * COO_WARPS) k_coo_rows(const int32_t* __re
 }
 
 cudaError_t build_schedule(const int32_t* rowptr, int64_t M, int64_t nnz, int32_t W, char* storage,
-                           const SchedLayout& L, int64_t* npieces_out, cudaStream_t s)
+                           const SchedLayout& L, int64_t* npieces_out, bool* regular_out, cudaStream_t s)
 {
     int32_t* rowidx = reinterpret_cast<int32_t*>(storage + L.rowidx);
     int2* bnd = reinterpret_cast<int2*>(storage + L.bnd);
@@ -291,21 +300,22 @@ cudaError_t build_schedule(const int32_t* rowptr, int64_t M, int64_t nnz, int32_
 
     if (M > 0 && nnz > 0) {
         const int64_t warps = (nnz + COO_SPAN - 1) / COO_SPAN;
-        k_coo_rows<<<(unsigned)((warps * 32 + 255) / 256), 256, 0, s>>>(rowptr, M, nnz, rowidx);
+        k_coo_rows<<<(unsigned)((warps * 32 + 255) / 256), 256, 0, s>>>(rowptr, M, nnz, rowidx, pieces + nc + 1);
     }
     k_sched_bounds<<<gb, 256, 0, s>>>(rowptr, M, nnz, W, nc, bnd, 0);
-    k_sched_pieces<<<gb, 256, 0, s>>>(bnd, rowptr, M, nc, pieces);
+    k_sched_pieces<<<gb, 256, 0, s>>>(bnd, rowptr, M, nnz, nc, pieces);
     cudaError_t err = scan_exclusive_i32(pieces, pieces, nc + 1, storage + L.scan_tmp, s);
     if (err != cudaSuccess) return err;
     k_sched_meta<<<gb, 256, 0, s>>>(bnd, rowptr, M, nc, pieces, meta, head_s0, slot_np, cnt);
     err = cudaGetLastError();
     if (err != cudaSuccess) return err;
-    int32_t np = 0;
-    err = cudaMemcpyAsync(&np, pieces + nc, sizeof(int32_t), cudaMemcpyDeviceToHost, s);
+    int32_t np[2] = {0, 1};                                          // pieces of split rows, whether rows differ in length
+    err = cudaMemcpyAsync(np, pieces + nc, (nnz > 0 ? 2 : 1) * sizeof(int32_t), cudaMemcpyDeviceToHost, s);
     if (err != cudaSuccess) return err;
     err = cudaStreamSynchronize(s);
     if (err != cudaSuccess) return err;
-    *npieces_out = np;
+    *npieces_out = np[0];
+    *regular_out = np[0] == 0 && np[1] == 0;
     return cudaSuccess;
 }
 

@@ -139,6 +139,31 @@ def test_empty_rows_of_16_bit_outputs(spk, odt):
     assert torch.equal(H, C.to(odt))
 
 
+def _rows_of(spk, M, d, seed=3):
+    """M rows of exactly d entries, uniform columns."""
+    g = torch.Generator(device=DEV).manual_seed(seed)
+    rp = (torch.arange(M + 1, device=DEV) * d).int()
+    ci = torch.randint(M, (M * d,), generator=g, device=DEV).int()
+    return spk.CSR(rp, ci, (M, M), torch.rand(M * d, generator=g, device=DEV))
+
+
+@pytest.mark.parametrize("K", [4, 12, 16])
+def test_narrow_rows_on_regular_patterns(spk, K):
+    """FP32 rows of up to 64 bytes, 8M entries, 24 a row: as fast as the row-split kernel (the warp kernel took twice
+    its time), and the bits of the balanced register path in every form that a call can have."""
+    S = _rows_of(spk, 333_000, 24)
+    wide = torch.randn(S.N, K + 4, device=DEV)
+    B, v2, reg = wide[:, :K], torch.rand(S.nnz, device=DEV), {"variant": 3}
+    assert torch.equal(spk.spmm(S, B), spk.spmm(S, B, tune=reg))
+    assert torch.equal(spk.spmm(S, B, vals2=v2), spk.spmm(S, B, vals2=v2, tune=reg))
+    assert torch.equal(spk.spmm(S, B, out_dtype=torch.bfloat16), spk.spmm(S, B, out_dtype=torch.bfloat16, tune=reg))
+    C, D = torch.ones(S.M, K, device=DEV), torch.ones(S.M, K, device=DEV)
+    spk.spmm(S, B, out=C, accumulate=True)
+    spk.spmm(S, B, out=D, accumulate=True, tune=reg)
+    assert torch.equal(C, D)
+    assert _time(lambda: spk.spmm(S, B)) <= 1.25 * _time(lambda: spk.spmm(S, B, tune={"variant": 1}))
+
+
 def test_spmm_t_with_two_value_arrays(spk):
     """2.5M entries, 25 a row, FP32 K = 64: a second array doubles what competes with the rows for L2 when both are
     gathered through the permutation (1.6 times the time of one array); put in order first they take 1.37 times."""
