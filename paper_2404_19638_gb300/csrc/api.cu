@@ -676,6 +676,18 @@ extern "C" spk_status spk_spmm_mh(spk_csr S, const float* vals, int64_t hstride,
 // ----------------------------------------------------------------------------
 extern "C" spk_status spk_fusedmm_workspace_size(spk_csr S, int32_t K, int32_t heads, size_t* bytes)
 {
+// One head, FP32, K = 64: time of the warp kernel over that of 8 lanes x 2
+// vectors, plain / softmax.  Rows of one length: 24 a row, 1M entries 0.5, 3M 1.16
+// / 1.19, 8M 1.21 / 1.28, 14M 1.29 / 1.36; 16 a row 3M 1.21 / 1.22, 8M 1.30 / 1.32;
+// 8 a row 3M 1.18 / 1.20, 8M 1.19 / 1.25, 14M 0.99 / 1.07; 4 a row 0.89-1.09; 24 but
+// for one row in 2000 14M 1.23 / 1.30.  Two lengths: 20 or 21 a row 8M 1.14 / 1.18,
+// 12M 0.98 / 1.03; 30 or 31 14M 1.07 / 1.13; 12 or 13 2.4M 0.69; 8 or 9 8.5M 0.82.
+// B of 12.8 MB, which stays near: 10M 0.96 / 0.99.  Random lengths 0.5-0.9, R-MAT 0.57-0.71.
+static bool fused_lanes_pay(const spk_csr_s* S, int K)
+{
+    return S->regular && S->nnz >= 5 << 19 && S->N * K * 4 >= 16 << 20 && S->nnz >= (S->nnz % S->M == 0 ? 6 : 12) * S->M;
+}
+
     REQUIRE(S && bytes && K >= 1 && heads >= 1, SPK_ERR_ARG, "spk_fusedmm_workspace_size: bad argument");
     *bytes = S->has_sched ? (size_t)S->npieces * (((size_t)K + 2 * (size_t)heads + 3) / 4 * 4) * 4 : 0;
     return SPK_OK;
@@ -712,7 +724,9 @@ extern "C" spk_status spk_fusedmm(spk_csr S, const float* vals, float scale, int
     // a power of two 16-byte vectors.  It was the faster one at every width,
     // head count and dtype measured (R-MAT of 8M nonzeros and 5 nonzeros a row,
     // K = 16-128, 1-4 heads; narrowest margin FP32 K = 128 in 4 heads at 5 a
-    // row: 0.277 against 0.313 ms).  Wider rows and other heads run one head per
+    // row: 0.277 against 0.313 ms), but for FP32 rows of 64 with one head on large
+    // patterns of rows of nearly one length, where the lane groups of a warp change
+    // rows together (fused_lanes_pay).  Wider rows and other heads run one head per
     // grid row, and so does a shape that is asked for; tune.vecs_per_lane alone
     // (no group_lanes, no unroll) asks for the lane-group kernel of all heads
     // with that many vectors a lane (1 or 2).
@@ -727,7 +741,8 @@ extern "C" spk_status spk_fusedmm(spk_csr S, const float* vals, float scale, int
                 SPK_ERR_UNSUPPORTED, "spk_fusedmm: %d vectors a row do not split into %d heads of %d-vector lanes", nv,
                 heads, mh_nv);
     }
-    const bool warp = !shaped && !mh_asked && fused_warp_supported(dt, K, heads);
+    const bool warp = !shaped && !mh_asked && fused_warp_supported(dt, K, heads) &&
+                      !(one_head && dt == SPK_F32 && fused_lanes_pay(S, K));
     const bool mh = mh_asked;
     int G, NV = 1, U = 4, idx = -1;
     if (!mh && !warp) {
