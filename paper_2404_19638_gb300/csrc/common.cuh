@@ -320,11 +320,10 @@ struct SpmmArgs {
     int64_t nchunks;
 };
 
-// exp(e - m) for a score e and the largest score m of its row so far.  A score
-// of -inf (an entry masked through its value) weighs nothing, also where all
-// scores so far are -inf and m with them: the difference would be NaN there and
-// stay in the row's sum.
-__device__ __forceinline__ float softmax_weight(float e, float m) { return e == -INFINITY ? 0.f : expf(e - m); }
+// What a softmax subtracts from scores whose maximum so far is m: m, or 0 where
+// all of them are -inf (entries masked through their value).  They weigh nothing
+// then; -inf - -inf would be NaN and stay in the row's sum.
+__device__ __forceinline__ float softmax_base(float m) { return m == -INFINITY ? 0.f : m; }
 
 // FusedMM: SDDMM cascaded into SpMM on one dense matrix B, per head of
 // heads equal slices of K (dh = K / heads): scores e = scale * s * <a_i, b_j>

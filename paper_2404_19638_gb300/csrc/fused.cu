@@ -357,9 +357,10 @@ __device__ __forceinline__ void fused_span(const FusedArgs& a, const Group<G>& g
                     const float c = (m == -INFINITY) ? 0.f : expf(m - mb);
                     rescale(c);
                     l *= c;
+                    const float base = softmax_base(mb);
 #pragma unroll
                     for (int u = 0; u < U; ++u) {
-                        const float w = softmax_weight(ev[u], mb);
+                        const float w = expf(ev[u] - base);
                         l += w;
                         accumulate(sl, u, w);
                     }
@@ -405,7 +406,7 @@ __device__ __forceinline__ void fused_span(const FusedArgs& a, const Group<G>& g
                         const float mb = fmaxf(m, ev[u]);
                         const float c = (m == -INFINITY) ? 0.f : expf(m - mb);
                         rescale(c);
-                        const float w = softmax_weight(ev[u], mb);
+                        const float w = expf(ev[u] - softmax_base(mb));
                         l = l * c + w;
                         accumulate(sl, u, w);
                         m = mb;
@@ -736,9 +737,10 @@ __device__ __forceinline__ void fused_span_mh(const FusedArgs& a, const Group<G>
 #pragma unroll
                     for (int q = 0; q < W; ++q) acc[q] *= c;
                     l *= c;
+                    const float base = softmax_base(mb);
 #pragma unroll
                     for (int u = 0; u < U; ++u) {
-                        const float w = softmax_weight(ev[u], mb);
+                        const float w = expf(ev[u] - base);
                         l += w;
                         float bf[W];
                         unpack_v(sl + u * NV * 32, bf);     // re-read: keeps U rows out of registers
@@ -796,7 +798,7 @@ __device__ __forceinline__ void fused_span_mh(const FusedArgs& a, const Group<G>
                         const float c = (m == -INFINITY) ? 0.f : expf(m - mb);
 #pragma unroll
                         for (int q = 0; q < W; ++q) acc[q] *= c;
-                        const float w = softmax_weight(ev[u], mb);
+                        const float w = expf(ev[u] - softmax_base(mb));
                         l = l * c + w;
                         axpy_pairs<W>(acc, w, bf);
                         m = mb;

@@ -424,7 +424,7 @@ __device__ __forceinline__ void fused_warp_span(const FusedArgs& a, unsigned cha
                         if (!upto) M = fmaxf(M, mo);
                         M = __shfl_sync(0xffffffffu, M, se, U);
                     }
-                    s = softmax_weight(s, M);
+                    s = expf(s - softmax_base(M));
                     float sum = s;
                     if (m == 0) {
 #pragma unroll

@@ -62,3 +62,23 @@ def test_masked_entries_weigh_nothing(spk, dt, heads, tune, fill):
             e = b @ a
             assert abs(lse[r, h] - torch.logsumexp(e, 0)) <= ATOL
             assert (y - torch.softmax(e, 0) @ b).abs().max() <= ATOL
+
+
+@pytest.mark.parametrize("bad", [np.nan, np.inf])
+@pytest.mark.parametrize("tune", [None, {"group_lanes": 8, "vecs_per_lane": 2, "unroll": 4}, {"vecs_per_lane": 1}])
+def test_rows_with_a_nan_or_infinite_score_are_zeros(spk, bad, tune):
+    """Such a row has no softmax: zeros, with an lse of -inf, in short, long and split rows; the others are untouched."""
+    K, N, lens = 64, 900, [1, 5, 16, 40, 300, 700] * 2
+    rng = np.random.default_rng(1)
+    rp = np.cumsum([0] + lens).astype(np.int32)
+    ci = np.concatenate([np.sort(rng.choice(N, n, replace=False)) for n in lens]).astype(np.int32)
+    A, B = (torch.from_numpy(rng.uniform(0.3, 0.6, (n, K)).astype(np.float32)).to(DEV) for n in (len(lens), N))
+    vals = np.ones(ci.size, np.float32)
+    run = lambda: spk.fusedmm(spk.CSR(rp, ci, (len(lens), N), torch.from_numpy(vals), device=DEV, chunk_work=96), A, B,
+                              softmax=True, want_lse=True, tune=tune)
+    Y0, _, l0 = run()
+    for r in range(6):
+        vals[rp[r] + rng.integers(lens[r])] = bad
+    Y, _, lse = run()
+    assert not Y[:6].any() and (lse[:6] == -np.inf).all()
+    assert torch.equal(Y[6:], Y0[6:]) and torch.equal(lse[6:], l0[6:])
