@@ -554,6 +554,11 @@ extern "C" spk_status spk_spmm_workspace_size(spk_csr S, int32_t K, size_t* byte
 
 // 16-byte vectors throughout: whole vectors a row, aligned rows of B and C.
 static bool spmm_vec(spk_dtype dtb, const void* B, int64_t ldb, int32_t K, spk_dtype dtc, const void* C, int64_t ldc)
+{
+    return (K % vec_elems(dtb)) == 0 && aligned16(B) && aligned16(C) && (ldb * dt_bytes(dtb)) % 16 == 0 &&
+           (ldc * dt_bytes(dtc)) % 16 == 0;
+}
+
 // Whether FP32 rows of at most 64 bytes run row-split instead of the balanced
 // warp kernel, which has work for half its lanes or fewer there.  Where all rows
 // are nearly of one length the split balances by itself and the lane groups of a
@@ -565,11 +570,6 @@ static bool spmm_vec(spk_dtype dtb, const void* B, int64_t ldb, int32_t K, spk_d
 static bool spmm_row_split_pays(const spk_csr_s* S, int dt, int K)
 {
     return dt == SPK_F32 && K <= 16 && S->regular && !S->vperm && S->nnz >= 6 << 20 && S->nnz >= 12 * S->M;
-}
-
-{
-    return (K % vec_elems(dtb)) == 0 && aligned16(B) && aligned16(C) && (ldb * dt_bytes(dtb)) % 16 == 0 &&
-           (ldc * dt_bytes(dtc)) % 16 == 0;
 }
 
 static spk_status spmm_common(const char* name, const spk_csr_s* S, const float* vals, const float* vals2,
@@ -629,16 +629,16 @@ static spk_status spmm_common(const char* name, const spk_csr_s* S, const float*
     a.heads = heads;
     a.hstride = hstride;
     a.B = B; a.ldb = ldb; a.b_scale = b_scale;
-    if (vec && L.ring && heads == 1 && spmm_row_split_pays(S, dtb, K)) {
-        a.bnd = nullptr;
-        L.chunks = L.ring = false;
-        L.shape = shape_index(4, 1, 4);
-    }
     a.C = C; a.ldc = ldc; a.dtc = dtc; a.accumulate = accumulate;
     a.bnd = L.chunks ? S->bnd : nullptr;
     a.meta = S->meta; a.head_s0 = S->head_s0; a.slot_np = S->slot_np; a.cnt = S->cnt;
     a.carry = reinterpret_cast<float*>(ws);
     a.nchunks = S->nchunks;
+    if (vec && L.ring && heads == 1 && spmm_row_split_pays(S, dtb, K)) {
+        a.bnd = nullptr;
+        L.chunks = L.ring = false;
+        L.shape = shape_index(4, 1, 4);
+    }
     int cb = vec || !L.ring ? 0 : part_bytes(dtb, B, ldb, K);
     if (cb && !part_spmm_pays(dtb, cb, K, S->nnz, S->npieces > 0)) cb = 0;
     cudaError_t e = cb ? launch_spmm_part(dtb, cb, a, stream) : launch_spmm(dtb, L, a, stream);
@@ -676,6 +676,11 @@ extern "C" spk_status spk_spmm_mh(spk_csr S, const float* vals, int64_t hstride,
 // ----------------------------------------------------------------------------
 extern "C" spk_status spk_fusedmm_workspace_size(spk_csr S, int32_t K, int32_t heads, size_t* bytes)
 {
+    REQUIRE(S && bytes && K >= 1 && heads >= 1, SPK_ERR_ARG, "spk_fusedmm_workspace_size: bad argument");
+    *bytes = S->has_sched ? (size_t)S->npieces * (((size_t)K + 2 * (size_t)heads + 3) / 4 * 4) * 4 : 0;
+    return SPK_OK;
+}
+
 // One head, FP32, K = 64: time of the warp kernel over that of 8 lanes x 2
 // vectors, plain / softmax.  Rows of one length: 24 a row, 1M entries 0.5, 3M 1.16
 // / 1.19, 8M 1.21 / 1.28, 14M 1.29 / 1.36; 16 a row 3M 1.21 / 1.22, 8M 1.30 / 1.32;
@@ -686,11 +691,6 @@ extern "C" spk_status spk_fusedmm_workspace_size(spk_csr S, int32_t K, int32_t h
 static bool fused_lanes_pay(const spk_csr_s* S, int K)
 {
     return S->regular && S->nnz >= 5 << 19 && S->N * K * 4 >= 16 << 20 && S->nnz >= (S->nnz % S->M == 0 ? 6 : 12) * S->M;
-}
-
-    REQUIRE(S && bytes && K >= 1 && heads >= 1, SPK_ERR_ARG, "spk_fusedmm_workspace_size: bad argument");
-    *bytes = S->has_sched ? (size_t)S->npieces * (((size_t)K + 2 * (size_t)heads + 3) / 4 * 4) * 4 : 0;
-    return SPK_OK;
 }
 
 extern "C" spk_status spk_fusedmm(spk_csr S, const float* vals, float scale, int32_t softmax, spk_dtype dt,
@@ -1229,6 +1229,7 @@ extern "C" spk_status spk_spmm_t_workspace_size(spk_tplan P, int32_t K, size_t* 
 //     row, 0.51 / 0.33 ms), R-MAT 4M 1.14, 16M 1.36
 //   rows of 128 bytes: 16M, 24 a row, 149 MB 1.28; 8M, 75 MB 0.96; 64 bytes: 16M,
 //     8 a row, 192 MB 1.37; 107 MB 1.05; 48-96 MB 0.88-0.99; 32 bytes: 0.83-1.0
+//   two arrays, 2.5M, 25 a row, K = 64, 46 MB: 90 / 77 us (one array 56 / 68)
 //   the same with split rows in S^T (R-MAT 4M-30M, a few hot rows): 0.81-0.96
 static bool spmm_t_gathers_values(const spk_tplan_s* P, int arrays, spk_dtype dty, const void* Y, int64_t ldy, int32_t K,
                                   spk_dtype dtx, const void* X, int64_t ldx, const spk_tune* tune)
@@ -1259,7 +1260,6 @@ extern "C" spk_status spk_spmm_t(spk_tplan P, const float* vals, const float* va
     // every argument check of the SpMM on S^T runs before the value permutation
     spk_status st = spmm_common("spk_spmm_t", &P->St, (vals || vals2) ? reinterpret_cast<const float*>(w) : nullptr,
                                 nullptr, dty, Y, ldy, y_scale, K, dtx, X, ldx, accumulate, w ? w + vb : nullptr,
-//   two arrays, 2.5M, 25 a row, K = 64, 46 MB: 90 / 77 us (one array 56 / 68)
                                 w ? ws_bytes - vb : 0, tune, (cudaStream_t)stream, true, true);
     if (st != SPK_OK) return st;
     // The balanced 16-byte vector path can gather the values through the
