@@ -80,7 +80,7 @@ def peaks():
     return dict(FALLBACK_PEAKS), "fallback"
 
 
-# The files the step kernels (k_sddmm_ring, k_spmm_ring and their register
+# The files the step kernels (k_sddmm_warp, k_spmm_warp and their register
 # and row-split siblings) compile from: a change elsewhere in csrc/ (FusedMM,
 # batch, tensor-core tiles, plans) leaves their ncu traffic valid.
 STEP_KERNEL_SOURCES = ("common.cuh", "tiles.cuh", "lean.cuh", "ring.cuh", "rows.cuh", "sddmm_impl.cuh", "spmm_impl.cuh",

@@ -356,17 +356,12 @@ enum { OP_SDDMM = 0, OP_SPMM = 1, OP_SPMM_T = 2 };
 // Default lane-group shape for a row of nvec 16-byte vectors, from shape
 // sweeps on GB300 with the L2 flushed before each launch (R-MAT scale 20 and
 // 22 with K = 64, the K = 128 Chung-Lu pattern of 50M nonzeros):
-//   SDDMM: 4 lanes x 2 vectors at 8 vectors a row, 8 lanes x 2 vectors at 16,
-//          8 lanes x 4 vectors at 32, 4 nonzeros in flight;
-//   SpMM (and S^T Y): one vector a lane on 16 lanes with 8 nonzeros in
-//          flight at 16 vectors; 16 lanes x 2 vectors x 8 at 32 (rec FP32
-//          1.90 ms against 2.24 for 8 x 4 x 4).  16-bit rows of 8 vectors
-//          spread over 16 lanes as 8-byte vectors (8 nonzeros in flight) when
-//          rows are long (rmat20, 15 nonzeros a row: 0.412 ms), else 8 lanes
-//          of 16-byte vectors with 4 in flight (R-MAT scale 22, 8 a row:
-//          0.803 ms against 0.867); 16-bit rows of 16 vectors take 8 lanes x
-//          2 vectors x 4 (rec BF16 1.26 ms against 1.58 for 32 lanes of
-//          8-byte vectors).
+//   SDDMM (warp kernel): 4 lanes x 2 vectors at 8 vectors a row, 8 lanes x 2
+//          vectors at 16, 8 lanes x 4 vectors at 32, 4 nonzeros in flight.
+//   SpMM (and S^T Y) of variants 1 and 3; the warp kernel of variant 2 has one
+//          layout per row width and no shape: one vector a lane, 8 nonzeros in
+//          flight at 16 vectors, 16 lanes x 2 vectors x 8 at 32.  The shapes of
+//          16-bit rows (half16, short_rows) are only what variant 2 reports.
 static void default_shape(int op, int nvec, int* G, int* NV, int* U, bool half16 = false, bool short_rows = false)
 {
     *U = 4;

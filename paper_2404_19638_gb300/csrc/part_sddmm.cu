@@ -1,6 +1,6 @@
 // SDDMM on rows that 16 bytes do not divide.  8-byte copies are compiled for
-// FP32 pairs only (K even is the usual ragged width); the rest goes 4 bytes at
-// a time.
+// FP32 pairs only, where they cover every even K; in 16 bits they need K to be
+// a multiple of 4, and K = 100 takes 4-byte copies like the other even widths.
 #include "part.cuh"
 #include "sddmm_warp.cuh"
 

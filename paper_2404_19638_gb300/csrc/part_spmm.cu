@@ -1,4 +1,5 @@
 // SpMM on rows that 16 bytes do not divide (outputs of any dtype and mode).
+// 8-byte copies are compiled for FP32 only (see part_sddmm.cu).
 #include "part.cuh"
 #include "spmm_warp.cuh"
 

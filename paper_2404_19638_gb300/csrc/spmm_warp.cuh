@@ -32,11 +32,11 @@
 // row, FP32, K = 50).
 //
 // What bounds it (GB300, R-MAT scale 20, 16.1M nonzeros, K = 64): the
-// shared-memory data path, 75 % busy in FP32 (each gathered row is written and
+// shared-memory data path, 83 % busy in FP32 (each gathered row is written and
 // read once there), and instruction issue for 16-bit rows (the widening).
-// Measured, lane-group ring before / this: FP32 0.399 / 0.306 ms, BF16 0.407 /
-// 0.232 ms; BF16 K = 128 on the 50M-nonzero bipartite pattern 1.20 / 0.96 ms;
-// R-MAT scale 22 BF16 K = 64 0.775 / 0.554 ms.  Register gathers with one
+// Measured, lane-group ring before / this: FP32 0.399 / 0.282 ms, BF16 0.407 /
+// 0.220 ms; BF16 K = 128 on the 50M-nonzero bipartite pattern 1.20 / 0.87 ms;
+// R-MAT scale 22 BF16 K = 64 0.775 / 0.513 ms.  Register gathers with one
 // chunk per lane group and the same row masks: 0.36 / 0.35 ms (too few bytes
 // in flight at 28 warps a SM).  Batches of 16 rows up to 256 bytes, 8 above:
 // K = 128 FP32 0.49 ms with 8, 0.58 with 16 (half the warps fit); 16-bit

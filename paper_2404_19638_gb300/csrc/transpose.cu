@@ -5,9 +5,9 @@
 //
 // Built by a stable least-significant-digit radix sort of (column, nonzero
 // index) pairs, 8 bits per pass: per-tile digit histograms, one exclusive scan
-// over the digit-major histogram table, and a scatter that ranks equal digits
-// inside a tile in index order (warp match + per-warp digit counts), so that
-// rows stay ascending inside every column.
+// over the digit-major histogram table, and a scatter in which every warp ranks
+// its items on its own in index order (ballots and per-warp digit counts), so
+// that rows stay ascending inside every column.
 #include "common.cuh"
 
 namespace spk {
