@@ -167,17 +167,18 @@ __device__ __forceinline__ void chunk_flags(const int2* bnd, const int32_t* rowp
 }
 
 // pieces[nchunks + 1] is set where some boundary lies off the line on which it
-// would lie if all rows had one length, by more than a tenth of sqrt(nnz) entries
-// (random row lengths come several times as far), so that kernels whose lane
-// groups take rows of their own can tell patterns on which they keep in step.
-__global__ void k_sched_pieces(const int2* bnd, const int32_t* rowptr, int64_t M, int64_t nnz, int64_t nchunks,
-                               int32_t* pieces)
+// would lie if all rows had the mean length, by more than tol = a tenth of
+// sqrt(nnz) entries (random row lengths come several times as far), so that
+// kernels whose lane groups take rows of their own can tell patterns on which
+// they keep in step.
+__global__ void k_sched_pieces(const int2* bnd, const int32_t* rowptr, int64_t M, double mean, double tol,
+                               int64_t nchunks, int32_t* pieces)
 {
     const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (c > nchunks) return;
-    if (nnz > 0) {
+    if (mean > 0.0) {
         const int r = bnd[c].x;
-        if (fabs((double)rowptr[r] - (double)r * (double)nnz / (double)M) > 0.1 * sqrt((double)nnz)) pieces[nchunks + 1] = 1;
+        if (fabs(fma(-mean, (double)r, (double)rowptr[r])) > tol) pieces[nchunks + 1] = 1;
     }
     if (c == nchunks) { pieces[c] = 0; return; }
     int head, tail, r_last;
@@ -303,7 +304,7 @@ cudaError_t build_schedule(const int32_t* rowptr, int64_t M, int64_t nnz, int32_
         k_coo_rows<<<(unsigned)((warps * 32 + 255) / 256), 256, 0, s>>>(rowptr, M, nnz, rowidx, pieces + nc + 1);
     }
     k_sched_bounds<<<gb, 256, 0, s>>>(rowptr, M, nnz, W, nc, bnd, 0);
-    k_sched_pieces<<<gb, 256, 0, s>>>(bnd, rowptr, M, nnz, nc, pieces);
+    k_sched_pieces<<<gb, 256, 0, s>>>(bnd, rowptr, M, M > 0 ? (double)nnz / (double)M : 0.0, 0.1 * sqrt((double)nnz), nc, pieces);
     cudaError_t err = scan_exclusive_i32(pieces, pieces, nc + 1, storage + L.scan_tmp, s);
     if (err != cudaSuccess) return err;
     k_sched_meta<<<gb, 256, 0, s>>>(bnd, rowptr, M, nc, pieces, meta, head_s0, slot_np, cnt);
